@@ -2,7 +2,8 @@
 
 A case is a dict of plain values; ``kind`` says which calls one pass makes:
 
-  lookup   one ``FlowTable.lookup`` (``refresh`` > 0: a timers table, hits restart their timer)
+  lookup   one ``FlowTable.lookup`` (``refresh`` > 0: a timers table, one batch per time unit,
+           and each hit restarts its flow's timer)
   host     one lookup whose keys and results stay in pinned host memory
   batched  one ``BatchedLookup.launch`` over a burst of keys for each of many tables
   cycle    new flows arrive, are looked up and leave: insert, lookup, delete on one table
@@ -185,7 +186,7 @@ def _filled(case: dict, seed: int, flows: int, timers: bool):
 def _prepare_lookup(case, seed):
     m = int(case["lf"] * SLOTS * case["nb"])
     table, fill = _filled(case, seed, m, case["refresh"] > 0)
-    return {"case": case, "table": table, "keys": _lookup_keys(seed, _lookups(case, seed, m), fill), "now": 1}
+    return {"case": case, "table": table, "keys": _lookup_keys(seed, _lookups(case, seed, m), fill), "now": 0}
 
 
 def _prepare_host(case, seed):
@@ -289,7 +290,10 @@ def run(state):
 
 
 def _run_lookup(s):
-    return s["table"].lookup(s["keys"], s["now"] if s["case"]["refresh"] else 0, s["case"]["refresh"])
+    refresh = s["case"]["refresh"]
+    if refresh:
+        s["now"] += 1
+    return s["table"].lookup(s["keys"], s["now"], refresh)
 
 
 def _run_host(s):
