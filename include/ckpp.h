@@ -276,10 +276,10 @@ int ckpp_bulk_insert(ckpp_table* table, const ckpp_key* keys, const uint64_t* va
  * launch their work; no counterpart in the paper, and the results are the
  * same either way. Modes:
  *   CKPP_INSERT_LAUNCH_CHAIN   (the default) a chain of dependent kernels:
- *                              duplicate resolution, the slot claims, their
- *                              publication, the one-move pass, three
- *                              cuckoo-path searches, the filter fixup, each
- *                              launched to start while its predecessor drains;
+ *                              duplicate resolution and the slot claims, the
+ *                              one-move pass, three cuckoo-path searches, the
+ *                              filter fixup, each launched to start while its
+ *                              predecessor drains;
  *   CKPP_INSERT_LAUNCH_SINGLE  one cooperative launch running the same stages
  *                              separated by grid-wide barriers, sized to the
  *                              batch, with stages that have nothing to do

@@ -247,7 +247,7 @@ int ckpp_batch_insert(ckpp_batch* b, const ckpp_key* keys, const uint32_t* table
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
   if (int rc = prepare_workspace(n, workspace, workspace_bytes, s, ws)) return rc;
-  const TableSet ts{b->host_views[0], b->dev_views, table_ids, (uint32_t)b->tables.size()};
+  const TableSet ts{b->host_views[0], b->dev_views, table_ids, (uint32_t)b->tables.size(), b->any_timers ? 1u : 0u};
   return cuda_rc(launch_insert(ts, reinterpret_cast<const uint8_t*>(keys), vals, n, now, (now + ttl) & 0xFFFFu, status,
                                ws, s));
 }
@@ -262,7 +262,7 @@ int ckpp_batch_delete(ckpp_batch* b, const ckpp_key* keys, const uint32_t* table
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
   if (int rc = prepare_workspace(n, workspace, workspace_bytes, s, ws)) return rc;
-  const TableSet ts{b->host_views[0], b->dev_views, table_ids, (uint32_t)b->tables.size()};
+  const TableSet ts{b->host_views[0], b->dev_views, table_ids, (uint32_t)b->tables.size(), b->any_timers ? 1u : 0u};
   return cuda_rc(launch_delete(ts, reinterpret_cast<const uint8_t*>(keys), n, now, status, ws, s));
 }
 

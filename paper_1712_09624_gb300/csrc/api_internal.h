@@ -33,40 +33,39 @@ inline bool geometry_ok(const ckpp_geometry* g) {
 
 inline size_t table_bytes(const ckpp_geometry* g) { return kHeaderBytes + (size_t)g->n_buckets * kBucketBytes; }
 
-// Workspace of an n-key batch: counters | set[2m] (first and last index per
-// position, interleaved) | slot_of[n] | dup[n] (bytes) | pending[n] | retry[n]
-// | claim[n] (8 bytes each) | fixup[fix_cap] (8 bytes each), each part
-// 256-byte aligned.
+// Workspace of an n-key batch: counters | set[m] | range[n] (8 bytes each) |
+// followers[n] (8) | pending[n] | retry[n] | sticky[n] (8) |
+// fixup[fix_cap] (8), each part 256-byte aligned.
 struct WsLayout {
   uint64_t m = 0;
-  uint32_t fix_cap = 0;
-  size_t off_set = 0, off_slot = 0, off_dup = 0, off_pending = 0, off_retry = 0, off_claim = 0, off_fixup = 0,
+  uint32_t idx_bits = 0, fix_cap = 0;
+  size_t off_set = 0, off_range = 0, off_followers = 0, off_pending = 0, off_retry = 0, off_sticky = 0, off_fixup = 0,
          total = 0;
 };
 
 constexpr WsLayout ws_layout(uint64_t n) {
   WsLayout L;
-  // The dedup set probes linearly, and its longest probe sequence (a dependent
-  // key read and CAS per step) sets the dedup kernel's time: at load 1/2 about
-  // 30 steps for 32K keys, at 1/8 about 7. So m is a power of two of at least
-  // 8n up to 2^17 keys (at most 8 MB of set) and 4n above (at most 2^32).
+  // The dedup set probes linearly, and a warp waits for the longest probe
+  // sequence of its lanes (a dependent CAS per step). So m is a power of two of
+  // at least 8n up to 2^17 keys (at most 4 MB of set) and 4n above (at most 2^32).
   uint64_t m = 64;
   const uint64_t want = n <= (1ull << 17) ? 8 * n : 4 * n;
   while (m < want) m <<= 1;
   L.m = m;
+  while ((1ull << L.idx_bits) <= n) ++L.idx_bits;  // so that no set word equals kEmpty
   L.fix_cap = (uint32_t)(n < (1ull << 22) ? n : (1ull << 22)) + 64;
-  size_t off = kAlign;  // counters
+  size_t off = align_up(4 * kCounterWords, kAlign);
   L.off_set = off;
-  off = align_up(off + 8 * m, kAlign);
-  L.off_slot = off;
-  off = align_up(off + 4 * n, kAlign);
-  L.off_dup = off;
-  off = align_up(off + n, kAlign);
+  off = align_up(off + 4 * m, kAlign);
+  L.off_range = off;
+  off = align_up(off + 8 * n, kAlign);
+  L.off_followers = off;
+  off = align_up(off + 8 * n, kAlign);
   L.off_pending = off;
   off = align_up(off + 4 * n, kAlign);
   L.off_retry = off;
   off = align_up(off + 4 * n, kAlign);
-  L.off_claim = off;
+  L.off_sticky = off;
   off = align_up(off + 8 * n, kAlign);
   L.off_fixup = off;
   off = align_up(off + 8 * (size_t)L.fix_cap, kAlign);
@@ -80,15 +79,16 @@ inline int prepare_workspace(uint64_t n, void* workspace, size_t bytes, cudaStre
   uint8_t* w = static_cast<uint8_t*>(workspace);
   ws.counters = reinterpret_cast<uint32_t*>(w);
   ws.set = reinterpret_cast<uint32_t*>(w + L.off_set);
-  ws.slot_of = reinterpret_cast<uint32_t*>(w + L.off_slot);
-  ws.dup = w + L.off_dup;
+  ws.range = reinterpret_cast<uint2*>(w + L.off_range);
+  ws.followers = reinterpret_cast<uint2*>(w + L.off_followers);
   ws.pending = reinterpret_cast<uint32_t*>(w + L.off_pending);
   ws.retry = reinterpret_cast<uint32_t*>(w + L.off_retry);
-  ws.claim = reinterpret_cast<unsigned long long*>(w + L.off_claim);
+  ws.sticky = reinterpret_cast<unsigned long long*>(w + L.off_sticky);
   ws.fixup = reinterpret_cast<unsigned long long*>(w + L.off_fixup);
   ws.m_mask = (uint32_t)(L.m - 1);
+  ws.idx_bits = L.idx_bits;
   ws.fix_cap = L.fix_cap;
-  return launch_workspace_clear(ws, (uint32_t)(kAlign / 4), n, s) == cudaSuccess ? CKPP_OK : CKPP_ECUDA;
+  return launch_workspace_clear(ws, s) == cudaSuccess ? CKPP_OK : CKPP_ECUDA;
 }
 
 // Sec. 4.2: a timed call more than 64512 units after the last scan could see
@@ -118,7 +118,7 @@ inline int residency(const void* p) {
 }
 
 // One table as a TableSet.
-inline TableSet one_table(const ckpp_table* t) { return TableSet{t->view, nullptr, nullptr, 1u}; }
+inline TableSet one_table(const ckpp_table* t) { return TableSet{t->view, nullptr, nullptr, 1u, t->view.timers}; }
 
 inline int check_keys(const ckpp_key* keys, uint64_t n) {
   if (n > kMaxBatch) return CKPP_EINVAL;

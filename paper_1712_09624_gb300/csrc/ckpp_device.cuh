@@ -101,8 +101,8 @@ __device__ __forceinline__ uint32_t reduce(uint64_t h, uint64_t nb) {
   return (uint32_t)(((h >> 32) * (uint64_t)(uint32_t)nb) >> 32);
 }
 
-__device__ __forceinline__ Addr address_of(const Key& k, uint64_t nb, uint64_t seed) {
-  const uint64_t h1 = hash_key(k, seed);
+__device__ __forceinline__ Addr address_of(const Key& k, uint64_t nb, uint64_t seed, uint64_t& h1) {
+  h1 = hash_key(k, seed);
   const uint64_t h2 = hash_key(k, seed ^ kSeed2Xor);
   Addr a;
   a.b1 = reduce(h1, nb);
@@ -111,6 +111,11 @@ __device__ __forceinline__ Addr address_of(const Key& k, uint64_t nb, uint64_t s
   a.tag = (uint32_t)(h1 & 0xFFFF);
   a.bits = (1ull << (h2 & 63)) | (1ull << ((h2 >> 6) & 63));
   return a;
+}
+
+__device__ __forceinline__ Addr address_of(const Key& k, uint64_t nb, uint64_t seed) {
+  uint64_t h1;
+  return address_of(k, nb, seed, h1);
 }
 
 // ---------------------------------------------------------- timers (Sec. 4.2)
@@ -230,6 +235,10 @@ __device__ __forceinline__ void st64_cg(void* p, uint64_t v) {
 __device__ __forceinline__ void st16_cg(void* p, uint32_t v) {
   asm volatile("st.global.relaxed.gpu.u16 [%0], %1;" ::"l"(p), "h"((uint16_t)v) : "memory");
 }
+
+// The 64-bit halves of a 16-byte vector.
+__device__ __forceinline__ uint64_t lo64(const uint4& v) { return (uint64_t)v.x | (uint64_t)v.y << 32; }
+__device__ __forceinline__ uint64_t hi64(const uint4& v) { return (uint64_t)v.z | (uint64_t)v.w << 32; }
 
 // Set a slot's expiry (timers tables only).
 __device__ __forceinline__ void set_expiry(const TableView& t, uint32_t b, uint32_t s, uint32_t expiry) {

@@ -31,31 +31,35 @@ inline int device_sm_count() {
   return v;
 }
 
-// Device scratch for one insert or delete batch (carved out of the caller's
-// workspace buffer, see workspace_layout in api.cu).
-struct Workspace {
-  uint32_t* counters;   // [0] pending count, [1] fixup count, [2] fixup overflow flag; list counts of the
-                        // displacement passes: [3] after move1 (in `retry`), [5] after the grid search
-                        // (in `pending`), [6] after the second search (in `retry`)
-  uint32_t* set;        // [2m] open-addressing set of batch keys; position p holds two words side by
-                        // side (one line for both): the lowest batch index of the key (kEmpty when
-                        // free) and the highest
-  uint32_t* slot_of;    // [n] set position of each batch key
-  uint8_t* dup;         // [n] 1 when the key's group has other members (cleared to 0 with the set)
-  uint32_t* pending;    // [n] leaders left for the displacement pass
-  uint32_t* retry;      // [n] leaders a displacement pass passes on to the next
-  unsigned long long* claim;  // [n] per key: (bucket << 32) | the ctrl bits its publication flips, or 0
-                              // (the slot phase 1 claimed for it; written by phase 1 for every key)
-  unsigned long long* fixup;  // [fix_cap] (table << 32 | bucket) whose moved counter fell to 0 off-lock
-  uint32_t m_mask;      // m - 1 (m a power of two >= 4n)
-  uint32_t fix_cap;
+// Words of a workspace's counters. The first 32 bytes are a caller's diagnostics
+// (ckpp_workspace_bytes): list counts of the displacement passes. Counters that
+// one kernel appends to are in lines of their own.
+constexpr uint32_t kCntPending = 0,    // keys phase 1 left (in `pending`)
+    kCntFixup = 1, kCntFixupOverflow = 2,
+                   kCntMoved1 = 3,     // keys the one-move pass left (in `retry`)
+    kCntGrid = 5,                      // keys the grid search left (in `pending`)
+    kCntSecond = 6,                    // keys the second search left (in `retry`)
+    kCntBarrier = 8,                   // two words: the grid barrier of the single-launch insert
+    kCntFollowers = 32, kCntSticky = 64;
+constexpr uint32_t kCounterWords = 128;
 
-  __device__ __forceinline__ uint32_t* first_at(uint32_t p) const { return set + 2 * (uint64_t)p; }
-  __device__ __forceinline__ uint32_t* last_at(uint32_t p) const { return set + 2 * (uint64_t)p + 1; }
-  // both words of position p as one 64-bit word: first in the low half, last in the high half
-  __device__ __forceinline__ unsigned long long* pair_at(uint32_t p) const {
-    return reinterpret_cast<unsigned long long*>(set + 2 * (uint64_t)p);
-  }
+// Device scratch for one insert or delete batch (carved out of the caller's
+// workspace buffer, see ws_layout in api_internal.h). Only the counters and the
+// set are cleared before a call; every other word is written before it is read.
+struct Workspace {
+  uint32_t* counters;   // list counts (kCnt*)
+  uint32_t* set;        // [m] open-addressing set of batch keys (dedup.cuh): hash bits << idx_bits | batch index of
+                        // the key that claimed the position, or kEmpty
+  uint2* range;         // [n] lowest and highest batch index of the group of key i, for groups with followers
+  uint2* followers;     // [n] (batch index, its group's owner): the keys that repeat another key of the batch
+  uint32_t* pending;    // [n] owners left for the displacement pass
+  uint32_t* retry;      // [n] owners a displacement pass passes on to the next
+  unsigned long long* sticky;  // [n] (batch index << 32 | bucket): buckets of timers tables whose claimed bits the
+                               // finishing pass clears
+  unsigned long long* fixup;   // [fix_cap] (table << 32 | bucket) whose moved counter fell to 0 off-lock
+  uint32_t m_mask;      // m - 1 (m a power of two >= 4n)
+  uint32_t idx_bits;    // bits of a batch index in a set word: n < 2^idx_bits
+  uint32_t fix_cap;
 };
 
 // The table(s) a mutation batch works on: one table, or many (key i goes to
@@ -65,6 +69,7 @@ struct TableSet {
   const TableView* views;  // nullptr: every key goes to `single`
   const uint32_t* tab;     // per-key table index when views != nullptr
   uint32_t n_tables;
+  uint32_t any_timers;     // some table has timers
 
   __device__ __forceinline__ bool valid(uint64_t i) const { return !views || tab[i] < n_tables; }
   __device__ __forceinline__ uint32_t id(uint64_t i) const { return views ? tab[i] : 0u; }
@@ -94,12 +99,9 @@ cudaError_t launch_batched_lookup(const TableView* tables, uint32_t n_tables, co
                                   int keys_per_warp, bool any_timers, uint32_t blocks, unsigned long long* ctrl,
                                   cudaStream_t s);
 
-// Resets a carved workspace for a new batch: counter_words counters to 0, the
-// dedup set's first-index words to empty and last-index words to 0 (one launch).
-cudaError_t launch_workspace_clear(const Workspace& ws, uint32_t counter_words, uint64_t n, cudaStream_t s);
-
-cudaError_t launch_dedup(const TableSet& ts, const uint8_t* keys, uint64_t n, const Workspace& ws,
-                         cudaStream_t s);
+// Resets a carved workspace for a new batch: the counters to 0, the set to empty
+// (one launch).
+cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s);
 
 // An insert call runs as a chain of kernels (the default) or as one
 // cooperative launch (insert.cu), whichever mode the caller picks.

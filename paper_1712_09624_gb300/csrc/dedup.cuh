@@ -1,0 +1,140 @@
+// In-batch duplicate keys of an insert or delete call. A batch has the result
+// of applying its keys one by one in index order, but equal keys are found
+// while the batch runs: an open-addressing set in the workspace gives each
+// group of equal keys one owner, the member that claims the group's position
+// first, whichever that is. The owner does the group's work on the table; the
+// other members (followers) are listed, and after the owners' kernels
+//   follower_ranges   gives each group with followers its lowest and highest
+//                     batch index, and
+//   the call's last kernel settles the group: the lowest index reports the
+//                     outcome, the others that of a repeated key, and an
+//                     insert stores the value of the highest index.
+// So a key that occurs once (nearly all of them) pays for one CAS, which its
+// owner issues together with the read of its bucket, and no later pass looks
+// at it. (A separate dedup kernel before the table kernels, with a claimed
+// position's first and last index side by side and a flag byte per key, took
+// 28 us of a 1M-key call and as much again in reads by the passes after it.)
+//
+// A set word is 4 bytes: the batch index in its low idx_bits and as many bits
+// of the key's hash as remain above it, so that a position held by another key
+// is passed over without reading that key (1M keys: 11 bits, one false match
+// in 2048).
+#pragma once
+
+#include "mutate.cuh"
+
+namespace ckpp {
+
+constexpr uint32_t kWarpAll = 0xFFFFFFFFu;
+constexpr uint32_t kNoIndex = 0xFFFFFFFFu;
+
+__device__ __forceinline__ Key load_key(const uint8_t* keys, uint64_t i) {
+  uint64_t a, b;
+  asm volatile("ld.global.nc.v2.u64 {%0,%1}, [%2];" : "=l"(a), "=l"(b) : "l"(keys + 16 * i));
+  return Key{a, b};
+}
+
+// The set word of batch key i (h1: its primary hash).
+__device__ __forceinline__ uint32_t set_word(const Workspace& ws, uint64_t h1, uint32_t i) {
+  return ((uint32_t)h1 >> ws.idx_bits << ws.idx_bits) | i;
+}
+
+// A key's probe of the set: its position, its word and what the CAS returned.
+struct SetProbe {
+  uint32_t pos, word, old;
+};
+
+// The first CAS (h1: the key's primary hash, tid: its table). Its result is
+// not looked at here, so that the caller can request more before waiting.
+__device__ __forceinline__ SetProbe set_probe(const Workspace& ws, uint64_t h1, uint32_t tid, uint32_t i) {
+  const uint64_t h = h1 ^ (uint64_t)tid * 0x9E3779B97F4A7C15ull;  // one key bound for many tables spreads out
+  SetProbe p;
+  p.pos = (uint32_t)(h >> 16) & ws.m_mask;
+  p.word = set_word(ws, h1, i);
+  p.old = atomicCAS(ws.set + p.pos, kEmpty, p.word);
+  return p;
+}
+
+// The owner of key i's group: i itself if a probe found a free position (the
+// set has 4n positions or more, so one is met). Equal keys bound for
+// different tables are different keys.
+__device__ __forceinline__ uint32_t set_owner(const Workspace& ws, const TableSet& ts, const uint8_t* keys,
+                                              const Key& k, uint32_t tid, uint32_t i, SetProbe p) {
+  for (uint32_t n = 0; n <= ws.m_mask; ++n) {
+    if (p.old == kEmpty) return i;
+    if (((p.old ^ p.word) >> ws.idx_bits) == 0u) {
+      const uint32_t cur = p.old & ((1u << ws.idx_bits) - 1u);
+      const Key o = load_key(keys, cur);
+      if (o.k0 == k.k0 && o.k1 == k.k1 && ts.id(cur) == tid) return cur;
+    }
+    p.pos = (p.pos + 1) & ws.m_mask;
+    p.old = atomicCAS(ws.set + p.pos, kEmpty, p.word);
+  }
+  return i;
+}
+
+// Appending to lists. Every returning atomic on one counter takes 0.8 ns (a
+// warp's append each, of a 1M-key batch: 26 us per list, and twice that for two
+// counters in one 128-byte line), so a block takes its places in all its lists
+// with one atomic per list, and the lists' counters are a line apart.
+template <int kLists>
+struct BlockLists {
+  uint32_t count[kLists], base[kLists];
+};
+
+// Before the first append (block-wide).
+template <int kLists>
+__device__ __forceinline__ void lists_init(BlockLists<kLists>& L) {
+  if (threadIdx.x < kLists) L.count[threadIdx.x] = 0;
+  __syncthreads();
+}
+
+// at[j] receives this thread's place in list j where want[j] (block-wide: every
+// thread of the block calls this).
+template <int kLists>
+__device__ __forceinline__ void lists_append(BlockLists<kLists>& L, uint32_t* const (&counters)[kLists],
+                                             const bool (&want)[kLists], uint32_t (&at)[kLists]) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (int j = 0; j < kLists; ++j) {
+    const uint32_t mask = __ballot_sync(kWarpAll, want[j]);
+    at[j] = 0;
+    if (mask) {
+      const uint32_t leader = __ffs(mask) - 1;
+      uint32_t first = 0;
+      if (lane == leader) first = atomicAdd(&L.count[j], (uint32_t)__popc(mask));
+      at[j] = __shfl_sync(kWarpAll, first, leader) + __popc(mask & ((1u << lane) - 1u));
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kLists; ++j) {
+    if (threadIdx.x == 32 * j && L.count[j]) {
+      L.base[j] = atomicAdd(counters[j], L.count[j]);
+      L.count[j] = 0;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kLists; ++j)
+    if (want[j]) at[j] += L.base[j];
+}
+
+// Key i as a follower of owner, at place at of the list. Each follower starts
+// its group's range at the owner (the same words from all).
+__device__ __forceinline__ void write_follower(const Workspace& ws, uint32_t at, uint32_t i, uint32_t owner) {
+  ws.followers[at] = make_uint2(i, owner);
+  ws.range[owner] = make_uint2(owner, owner);
+}
+
+// Widen each follower's group to include it (after the owners' kernel).
+__device__ __forceinline__ void follower_ranges(const Workspace& ws, uint32_t worker, uint32_t workers) {
+  const uint32_t count = ld32_cg(ws.counters + kCntFollowers);
+  for (uint32_t j = worker; j < count; j += workers) {
+    const uint2 f = ws.followers[j];
+    atomicMin(&ws.range[f.y].x, f.x);
+    atomicMax(&ws.range[f.y].y, f.x);
+  }
+}
+
+}  // namespace ckpp

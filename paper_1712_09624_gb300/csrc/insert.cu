@@ -2,20 +2,14 @@
 // counter upkeep; Sec. 4.2 reuse of dead slots).
 //
 // Kernels, in stream order:
-//   dedup   - groups equal keys of the batch in an open-addressing set in the
-//             workspace: each key learns the lowest (leader) and highest batch
-//             index of its group, which gives the batch the result of inserting
-//             the keys one by one in index order. Keys of groups with more than
-//             one member are flagged, so a key that occurs once needs no
-//             further read of the set.
-//   phase1  - per leader, lock-free: update in place if the key is stored
-//             (alive; a dead entry is revived), else claim the lowest free
-//             or dead slot of the primary, else of the secondary, with a CAS
-//             on the bucket's ctrl word, and write the entry into the
-//             claimed slot; leaders with two full buckets are queued for the
-//             displacement passes.
-//   publish - per key: the slot phase 1 claimed becomes busy (one atomic).
-//   move1   - per queued leader: the cuckoo paths of length one. Read the
+//   phase1  - per key, lock-free: the duplicate-key set (dedup.cuh) gives each
+//             group of equal keys one owner, which updates the key in place if
+//             it is stored (a dead entry is revived), else claims the lowest
+//             free or dead slot of the primary, else of the secondary, with a
+//             CAS on the bucket's ctrl word, writes the entry into the claimed
+//             slot and publishes it; owners with two full buckets are queued
+//             for the displacement passes.
+//   move1   - per queued owner: the cuckoo paths of length one. Read the
 //             entries of b1, then of b2, and the buckets they can move to; the
 //             first entry whose other bucket has a free or dead slot moves
 //             there under the locks of the path, and the key takes its slot.
@@ -31,14 +25,17 @@
 //             only then FULL.
 //   fixup and finish (one kernel) - reset the filter of buckets whose moved
 //             counter reached zero off their lock (the reset of Sec. 4.1,
-//             deferred so that it never races a concurrent setter); non-leader
-//             occurrences copy their leader's outcome (UPDATED, or FULL/BUSY).
-// Before them, one kernel clears the workspace (counters and the dedup set).
-// Each kernel after the workspace clear is launched with programmatic stream
-// serialization and waits for its predecessor in its first instruction
-// (pdl_wait in mutate.cuh), so the GPU schedules it while the predecessor
-// drains instead of after it.
-#include "mutate.cuh"
+//             deferred so that it never races a concurrent setter), clear the
+//             claimed bits that phase 1 left set in timers tables, and settle
+//             the groups of equal keys (the first occurrence reports the
+//             outcome, later ones UPDATED, or FULL/BUSY; the last one's value
+//             is stored), which gives the batch the result of inserting its
+//             keys one by one in index order.
+// Before them, one kernel clears the workspace (counters and the set). Each
+// kernel after it waits for its predecessor in its first instruction
+// (chain_launch.h).
+#include "chain_launch.h"
+#include "dedup.cuh"
 
 namespace ckpp {
 
@@ -49,137 +46,150 @@ constexpr int kPathAttempts = 16;
 // Buckets the one-move pass reads per round trip when looking for room for a root's entries.
 constexpr uint32_t kMoveGroup = 2;
 
-__device__ __forceinline__ Key load_key(const uint8_t* keys, uint64_t i) {
-  uint64_t a, b;
-  asm volatile("ld.global.nc.v2.u64 {%0,%1}, [%2];" : "=l"(a), "=l"(b) : "l"(keys + 16 * i));
-  return Key{a, b};
-}
-
-// ---------------------------------------------------------------- dedup
-// Equal keys bound for different tables are different keys.
-__device__ void dedup_one(const uint8_t* __restrict__ keys, const TableSet& ts, const Workspace& ws, uint64_t i) {
-  const Key k = load_key(keys, i);
-  const uint32_t tid = ts.id(i);
-  uint32_t pos = (uint32_t)(hash_key(k, 0x51ED270B27A2B5E3ull ^ tid) >> 16) & ws.m_mask;
-  const uint32_t me = (uint32_t)i;
-  constexpr unsigned long long kFreePair = kEmpty;  // first kEmpty, last 0
-  for (uint32_t probe = 0; probe <= ws.m_mask; ++probe) {
-    // one 64-bit CAS claims a free position (first = last = i) or returns the
-    // index range of the key group holding it
-    unsigned long long* pair = ws.pair_at(pos);
-    unsigned long long old = atomicCAS(pair, kFreePair, ((unsigned long long)me << 32) | me);
-    if (old == kFreePair) {
-      ws.slot_of[i] = pos;
-      return;
-    }
-    // A position only ever holds batch indices of one key group, so the key
-    // at index cur is that group's key even while other members widen the range.
-    const uint32_t cur = (uint32_t)old;
-    const Key o = load_key(keys, cur);
-    if (o.k0 == k.k0 && o.k1 == k.k1 && ts.id(cur) == tid) {
-      // widen the group's range to include i; a CAS fails only when another
-      // member's succeeded, so this ends within the group's size
-      for (;;) {
-        const uint32_t f = (uint32_t)old, l = (uint32_t)(old >> 32);
-        const unsigned long long want = ((unsigned long long)(l > me ? l : me) << 32) | (f < me ? f : me);
-        if (want == old) break;
-        const unsigned long long seen = atomicCAS(pair, old, want);
-        if (seen == old) break;
-        old = seen;
-      }
-      ws.slot_of[i] = pos;
-      // both occurrences are flagged: the first to claim the position learns of the
-      // group only here (every later occurrence's CAS returns a member of it)
-      ws.dup[i] = 1;
-      ws.dup[cur] = 1;
-      return;
-    }
-    pos = (pos + 1) & ws.m_mask;
-  }
-}
-
-__global__ void __launch_bounds__(kThreads) dedup_kernel(const uint8_t* __restrict__ keys, uint64_t n, TableSet ts,
-                                                         Workspace ws) {
-  pdl_wait();
-  pdl_release();
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i < n) dedup_one(keys, ts, ws, i);
-}
-
-// The first and last batch index of key i's group: i itself for a key that
-// occurs once in the batch (no read of the set), else one 8-byte read.
-__device__ __forceinline__ uint2 group_of(const Workspace& ws, uint64_t i) {
-  if (!ws.dup[i]) return make_uint2((uint32_t)i, (uint32_t)i);
-  return *reinterpret_cast<const uint2*>(ws.first_at(ws.slot_of[i]));
-}
-
-__device__ __forceinline__ bool is_leader(const Workspace& ws, uint64_t i, uint32_t& last) {
-  const uint2 g = group_of(ws, i);
-  if (g.x != (uint32_t)i) return false;
-  last = g.y;
-  return true;
-}
-
-// The value to store for key i: the last occurrence's of its group.
-__device__ __forceinline__ uint64_t value_of(const Workspace& ws, const uint64_t* vals, uint64_t i) {
-  return vals[group_of(ws, i).y];
-}
-
-// Status byte of a key that is not its group's first occurrence, until the
-// finishing pass copies its leader's outcome (never returned to the caller).
-constexpr uint8_t kStFollower = 0xFF;
-
 // --------------------------------------------------------------- phase 1
-// Per leader, without locks. A key that is stored (alive or dead, Sec. 4.2) is
-// found in its primary bucket, or in its secondary when the primary's filter
-// says it may be there (Sec. 4.1: a key stored in its secondary has both bits
-// set in its primary's filter; phase 1 moves no entry and the batch holds each
-// key once, so the tests are exact). A live entry is updated in place. Any
-// other key claims the lowest claimable slot of its primary, else of its
-// secondary (Sec. 2), else waits for the displacement passes.
+// Per key, without locks: the duplicate-key set (dedup.cuh) decides whether it
+// owns its group; an owner then finds its key or a slot for it.
+//
+// A key that is stored (alive or dead, Sec. 4.2) is found in its primary
+// bucket, or in its secondary when the primary's filter says it may be there
+// (Sec. 4.1: a key stored in its secondary has both bits set in its primary's
+// filter; phase 1 moves no entry and each key has one owner, so the tests are
+// exact). A live entry is updated in place. Any other key claims the lowest
+// claimable slot of its primary, else of its secondary (Sec. 2), else waits
+// for the displacement passes.
 //
 // A claim is a CAS on the bucket's ctrl word that sets the slot's claimed bit
 // (and clears its busy and in_secondary bits: a dead entry held there is
-// evicted, with moved-counter upkeep on its own primary). A slot is claimable
-// if it is neither busy nor claimed, or busy with a dead entry and not
-// claimed. The owner then writes the entry; the slot stays invisible to every
-// reader, whose searches look at busy slots only, until insert_publish (the
-// next kernel) flips its claimed bit to busy. A failed CAS returns the current
-// word, and the claimable slots are recomputed from it. Reviving a key's own
-// dead entry claims its slot in the same way (busy stays set), so a revival
-// and a reuse of that dead slot by another key cannot both succeed. Storing a
-// key in its secondary sets its two bits in the primary's filter and counts
-// it in the primary's moved counter, with relaxed atomics: no filter is reset
-// during phase 1 (resets of counters that reach zero here are deferred to the
-// fixup pass). Nothing in phase 1 waits on another thread, and nothing needs
-// a fence: the kernel boundary orders every write before the publication.
-constexpr int kClaimAttempts = 64;  // CAS retries on one bucket (at most 16 claims can change its word)
+// evicted, with moved-counter upkeep on its own primary). A failed CAS returns
+// the current word, and the claimable slots are recomputed from it. The owner
+// then writes the entry, and after a fence one atomic XOR turns the claimed
+// bit into busy: readers look at busy slots only, and one that meets a busy
+// slot with its key's tag reads the slot's key behind a fence of its own, so
+// it never sees the bytes that a freshly published slot held before.
+//
+// With timers two more rules keep a slot from being taken twice. A slot counts
+// as dead only if its expiry was read after (a fence) the ctrl word that
+// showed it busy; and a slot that held a dead entry keeps its claimed bit when
+// it is published (listed in ws.sticky, cleared by the finishing pass), since
+// its ctrl word would otherwise read as it did before the claim. Reviving a
+// key's own dead entry claims its slot in the same way (busy stays set), so a
+// revival and a reuse of that slot by another key cannot both succeed.
+//
+// Storing a key in its secondary sets its two bits in the primary's filter and
+// counts it in the primary's moved counter, with relaxed atomics: no filter is
+// reset during phase 1 (resets of counters that reach zero here are deferred
+// to the finishing pass). Nothing in phase 1 waits on another thread.
+//
+// What bounds it is the number of line requests, reads, writes and atomics
+// alike: on a 4 GiB buffer a thread per random line runs at 47 G/s with one
+// 32-byte read, at 24 with a store to the line after it, at 12 with three, and
+// at 8 with the whole sequence of a claim made by one thread (read, CAS, stores
+// of key, value and tag, XOR). Lanes that touch one line in one instruction
+// make one request together, so a warp gathers its keys' work: with timers the
+// header and the expiries come with one request (p1_fetch), and an entry's key
+// and value go out with one, its tag and expiry with another (p1_store).
+// Whole insert calls against separate dedup, claim and publication kernels that
+// made every request lane by lane: 1M keys into 134M slots at load 0.8 275 ->
+// 205 us, into 34M slots at 0.5 245 -> 175 us, with timers 280 -> 183 us; 64K
+// keys at 0.8 72 -> 65 us. (Taking exclusive ownership of a key's buckets in the
+// L2-resident set first, so that the table needs no atomics, was measured too:
+// 212 us where this takes 205, and slower with timers or with many keys per
+// bucket; the claims in the set cost what they save on the table.)
+constexpr int kClaimAttempts = 64;  // CAS retries on one bucket (two changes of its word per slot at most)
 
 __device__ __forceinline__ uint32_t claim_bit(uint32_t s) { return 1u << (kClaimShift + s); }
 
-// Slots of a bucket (ctrl word c, snapshot s) that an insertion may claim.
-__device__ __forceinline__ uint32_t claimable(const TableView& t, uint32_t c, const Snap& s, uint32_t now) {
-  return free_mask(t, c, s, now) & ~(c >> kClaimShift) & kBusyMask;
+// The slots that phase 1 may claim in a bucket whose word is c: free, or in
+// dead (busy slots found dead), and not claimed.
+__device__ __forceinline__ uint32_t claimable(uint32_t c, uint32_t dead) {
+  return (~c | dead) & ~(c >> kClaimShift) & kBusyMask;
 }
 
-// Claim the lowest claimable slot of bucket b. c: the word the snapshot s saw.
-// Returns the slot (prev receives the word the CAS replaced), -1 if nothing is
-// claimable, -2 after kClaimAttempts failed CASes.
-__device__ int claim_slot(const TableView& t, uint32_t b, uint32_t c, const Snap& s, uint32_t now, uint32_t& prev) {
-  uint32_t* cp = ctrl_ptr(t, b);
-  for (int i = 0; i < kClaimAttempts; ++i) {
-    const uint32_t f = claimable(t, c, s, now);
-    if (!f) return -1;
-    const uint32_t sl = __ffs(f) - 1;
-    const uint32_t want = (c | claim_bit(sl)) & ~((1u << sl) | (1u << (kInsecShift + sl)));
-    const uint32_t got = atomicCAS(cp, c, want);
-    if (got == c) {
-      prev = c;
-      return (int)sl;
+// A warp's rows in shared memory: the first 64 bytes of a bucket each, or a
+// store job each. 16-byte chunk c of row r is kept at c ^ (r >> 1 & 3).
+struct P1Rows {
+  unsigned long long addr[32];
+  __align__(128) uint4 row[32][4];
+};
+__device__ __forceinline__ uint4& row_chunk(P1Rows& R, uint32_t r, uint32_t c) { return R.row[r][c ^ ((r >> 1) & 3u)]; }
+
+// A bucket as phase 1 sees it.
+struct P1Bucket {
+  uint32_t b, ctrl, match;  // match: busy slots with the key's tag
+  uint32_t dead;            // busy slots with a dead entry (timers)
+  uint64_t bloom;
+};
+
+__device__ __forceinline__ P1Bucket p1_bucket(const TableView& t, uint32_t b, const Snap& s, uint32_t tag, bool timers,
+                                              uint32_t now) {
+  P1Bucket r;
+  r.b = b;
+  r.ctrl = (uint32_t)s.w[3];
+  r.match = tag_mask(s.w[0], s.w[1], tag) & r.ctrl & kBusyMask;
+  r.bloom = s.w[2];
+  r.dead = 0;
+  if (timers) {
+    r.dead = r.ctrl & ~alive_mask(s.e0, s.e1, now) & kBusyMask;
+    if (r.dead) {  // read again behind the ctrl word
+      fence_acq_rel();
+      uint64_t e0, e1;
+      ld128_cg(expiry_ptr(t, b, 0), e0, e1);
+      r.dead = r.ctrl & ~alive_mask(e0, e1, now) & kBusyMask;
     }
-    c = got;
   }
-  return -2;
+  return r;
+}
+
+// The header and (timers) the expiries of bucket b for every lane that wants
+// one (the whole warp calls this). With timers four lanes copy a bucket's first
+// 64 bytes together: reading them with two loads per lane is two requests.
+template <bool kTimers>
+__device__ __forceinline__ void p1_fetch(const TableView& t, uint32_t b, bool want, P1Rows& R, Snap& s) {
+  if (!kTimers) {
+    if (want) ld256_cg(bucket_ptr(t, b), s.w);
+    return;
+  }
+  const uint32_t lane = threadIdx.x & 31u, mask = __ballot_sync(kWarpAll, want);
+  if (!mask) return;
+  const uint32_t rank = __popc(mask & ((1u << lane) - 1u)), n = __popc(mask);
+  if (want) R.addr[rank] = reinterpret_cast<unsigned long long>(bucket_ptr(t, b));
+  __syncwarp();
+  for (uint32_t j = lane >> 2; j < n; j += 8) {
+    const uint32_t c = lane & 3u;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&row_chunk(R, j, c));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(R.addr[j] + 16u * c) : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  if (want) {
+    const uint4 a = row_chunk(R, rank, 0), h = row_chunk(R, rank, 1), e = row_chunk(R, rank, kExpiryOff / 16u);
+    s.w[0] = lo64(a), s.w[1] = hi64(a), s.w[2] = lo64(h), s.w[3] = hi64(h);
+    s.e0 = lo64(e), s.e1 = hi64(e);
+  }
+  __syncwarp();
+}
+
+// The same for one lane (rare).
+__device__ __forceinline__ void p1_fetch_one(const TableView& t, uint32_t b, bool timers, Snap& s) {
+  ld256_cg(bucket_ptr(t, b), s.w);
+  s.e0 = s.e1 = 0;
+  if (timers) ld128_cg(expiry_ptr(t, b, 0), s.e0, s.e1);
+}
+
+// The slot of bucket r holding key k, or -1.
+__device__ __forceinline__ int p1_find(const TableView& t, const P1Bucket& r, const Key& k) {
+  uint32_t cand = r.match;
+  if (!cand) return -1;
+  fence_acq_rel();
+  while (cand) {
+    const int slot = __ffs(cand) - 1;
+    cand &= cand - 1;
+    uint64_t k0, k1;
+    ld128_cg(key_ptr(t, r.b, slot), k0, k1);
+    if (k0 == k.k0 && k1 == k.k1) return slot;
+  }
+  return -1;
 }
 
 // Claim the slot of the key's own dead entry (slot sl of bucket b, busy in c).
@@ -196,156 +206,212 @@ __device__ int claim_revival(const TableView& t, uint32_t b, uint32_t sl, uint32
   return -2;
 }
 
-// A dead entry evicted by a claim (prev: the word before it): if it sat in its
-// secondary bucket, its primary's moved counter drops (Sec. 4.1); a counter
-// that reaches zero is queued for the filter reset of the fixup pass.
-__device__ __forceinline__ void evict_claimed(const TableView& t, uint32_t tid, uint32_t b, uint32_t sl,
-                                             uint32_t prev, const Workspace& ws) {
-  if (((prev >> sl) & 1u) && ((prev >> (kInsecShift + sl)) & 1u)) {
-    Key k;
-    ld128_cg(key_ptr(t, b, sl), k.k0, k.k1);
-    const Addr e = address_of(k, t.nb, t.seed);
-    if (atomicSub(moved_ptr(t, e.b1), 1u) == 1u) push_fixup(ws, tid, e.b1);
-  }
-}
+// What a key does with its slot.
+enum P1Work : uint32_t { kP1None, kP1Update, kP1Revive, kP1Place };
 
-struct P1Result {
-  uint8_t status;           // 0: queued for the displacement passes
-  unsigned long long rec;   // the claim to publish, or 0
-};
-
-// The key's stored entry in bucket b (snapshot s, word c), if any: a live one
-// is updated in place (UPDATED), a dead one revived through a claim
-// (INSERTED, Sec. 4.2). Returns false if the key is not there (or its dead
-// entry was just taken by another key).
-__device__ bool update_stored(const TableView& t, uint32_t b, uint32_t c, const Snap& s, const Key& k,
-                              const Addr& a, uint64_t v, uint32_t now, uint32_t expiry, P1Result& r) {
-  const int slot = find_key(t, b, c, s, k, a.tag);
-  if (slot < 0) return false;
-  if (!t.timers || alive16(snap_expiry(s, slot), now)) {
-    st64_cg(value_ptr(t, b, slot), v);
-    if (t.timers) set_expiry(t, b, slot, expiry);
-    r.status = kStUpdated;
-    return true;
-  }
-  const int got = claim_revival(t, b, (uint32_t)slot, c);
-  if (got == 0) return false;
-  if (got < 0) {
-    r.status = kStBusy;
-    return true;
-  }
-  st64_cg(value_ptr(t, b, slot), v);
-  set_expiry(t, b, slot, expiry);
-  r.status = kStInserted;
-  r.rec = ((unsigned long long)b << 32) | claim_bit(slot);
-  return true;
-}
-
-// Claim a slot of bucket b for the new key and write its entry there.
-// Returns false if b has nothing claimable.
-__device__ bool place_new(const TableView& t, uint32_t tid, uint32_t b, uint32_t c, const Snap& s, const Key& k,
-                          const Addr& a, uint64_t v, uint32_t now, uint32_t expiry, const Workspace& ws,
-                          P1Result& r) {
-  uint32_t prev = 0;
-  const int sl = claim_slot(t, b, c, s, now, prev);
-  if (sl == -1) return false;
-  if (sl < 0) {
-    r.status = kStBusy;
-    return true;
-  }
-  evict_claimed(t, tid, b, (uint32_t)sl, prev, ws);
-  st128_cg(key_ptr(t, b, sl), k.k0, k.k1);
-  st64_cg(value_ptr(t, b, sl), v);
-  st16_cg(tag_ptr(t, b, sl), a.tag);
-  if (t.timers) st16_cg(expiry_ptr(t, b, sl), expiry);
-  uint32_t flip = claim_bit(sl) | (1u << sl);
-  if (b == a.b2) {  // Sec. 4.1: displaced to the secondary
-    flip |= 1u << (kInsecShift + sl);
-    atomicOr(reinterpret_cast<unsigned long long*>(bloom_ptr(t, a.b1)), (unsigned long long)a.bits);
-    atomicAdd(moved_ptr(t, a.b1), 1u);
-  }
-  r.status = kStInserted;
-  r.rec = ((unsigned long long)b << 32) | flip;
-  return true;
-}
-
-__device__ void phase1_one(const TableSet& ts, const uint8_t* __restrict__ keys, const uint64_t* __restrict__ vals,
-                           uint32_t now, uint32_t expiry, uint8_t* __restrict__ status, const Workspace& ws,
-                           uint64_t i) {
-  P1Result r{0, 0ull};
-  // The leader test's set words and the primary's snapshot are independent
-  // round trips; both are requested before either is used.
-  const uint2 g = group_of(ws, i);
-  const uint32_t first = g.x, last = g.y;
-  if (!ts.valid(i)) {
-    ws.claim[i] = 0ull;
-    status[i] = first == (uint32_t)i ? kStNoTable : kStFollower;
-    return;
-  }
-  const TableView t = ts.of(i);
-  const uint32_t tid = ts.id(i);
-  const Key k = load_key(keys, i);
-  const Addr a = address_of(k, t.nb, t.seed);
-  Snap s1, s2;
-  snap_bucket(t, a.b1, s1);
-  if (first != (uint32_t)i) {
-    ws.claim[i] = 0ull;
-    status[i] = kStFollower;
-    return;
-  }
-  const uint64_t v = vals[last];
-  const uint32_t c1 = (uint32_t)s1.w[3];
-  bool done = update_stored(t, a.b1, c1, s1, k, a, v, now, expiry, r);
-  bool have2 = false;
-  uint32_t c2 = 0;
-  if (!done && (s1.w[2] & a.bits) == a.bits) {  // the filter allows the secondary
-    snap_bucket(t, a.b2, s2);
-    have2 = true;
-    c2 = (uint32_t)s2.w[3];
-    done = update_stored(t, a.b2, c2, s2, k, a, v, now, expiry, r);
-  }
-  if (!done) done = place_new(t, tid, a.b1, c1, s1, k, a, v, now, expiry, ws, r);
-  if (!done) {
-    if (!have2) {
-      snap_bucket(t, a.b2, s2);
-      c2 = (uint32_t)s2.w[3];
+// The key is stored in slot sl of bucket r: a live entry is updated in place
+// (UPDATED), a dead one revived through a claim (INSERTED, Sec. 4.2). Returns
+// the status, or 0 if the entry turned out to be a dead one that another key
+// has just taken.
+__device__ __forceinline__ uint8_t p1_stored(const TableView& t, const P1Bucket& r, uint32_t sl, bool timers,
+                                             P1Work& work) {
+  work = kP1Update;
+  if (timers) {
+    if ((r.dead >> sl) & 1u) {
+      const int got = claim_revival(t, r.b, sl, r.ctrl);
+      work = got > 0 ? kP1Revive : kP1None;
+      return got > 0 ? kStInserted : got == 0 ? 0 : kStBusy;
     }
-    done = place_new(t, tid, a.b2, c2, s2, k, a, v, now, expiry, ws, r);
+    // The expiry that called the entry alive may be that of a key which has taken
+    // the slot since: then the word shows its claim.
+    fence_acq_rel();
+    if ((ld32_cg(ctrl_ptr(t, r.b)) >> (kClaimShift + sl)) & 1u) {
+      work = kP1None;
+      return 0;
+    }
   }
-  ws.claim[i] = r.rec;
-  if (!done) {
-    ws.pending[atomicAdd(ws.counters + 0, 1u)] = (uint32_t)i;
-    return;
-  }
-  if (r.status == kStBusy) latch_error(t, kErrLockTimeout);
-  status[i] = r.status;
+  return kStUpdated;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) insert_phase1(TableSet ts, const uint8_t* __restrict__ keys,
-                                                          const uint64_t* __restrict__ vals, uint64_t n,
-                                                          uint32_t now, uint32_t expiry, uint8_t* __restrict__ status,
-                                                          Workspace ws) {
+// Claim the lowest claimable slot of bucket r. Returns the slot (prev receives
+// the word the CAS replaced), -1 if nothing is claimable, -2 after
+// kClaimAttempts failed CASes.
+__device__ __forceinline__ int claim_slot(const TableView& t, const P1Bucket& r, uint32_t& prev) {
+  uint32_t* cp = ctrl_ptr(t, r.b);
+  uint32_t c = r.ctrl;
+  for (int i = 0; i < kClaimAttempts; ++i) {
+    const uint32_t f = claimable(c, r.dead);
+    if (!f) return -1;
+    const uint32_t sl = __ffs(f) - 1;
+    const uint32_t want = (c | claim_bit(sl)) & ~((1u << sl) | (1u << (kInsecShift + sl)));
+    const uint32_t got = atomicCAS(cp, c, want);
+    if (got == c) {
+      prev = c;
+      return (int)sl;
+    }
+    c = got;
+  }
+  return -2;
+}
+
+// Store the warp's nj jobs. Row j of R: the key; the value and the bucket's
+// address; then which words to write (bits 0-5: the key's and the value's
+// four-byte words, 6 the tag, 7 the expiry) | slot << 8 | timers << 16, and
+// tag | expiry << 16. Six lanes store a job's key and value, two more its tag
+// and expiry in a second instruction (their neighbours belong to other keys'
+// claims, so they go out as 16-bit words).
+template <bool kTimers>
+__device__ __forceinline__ void p1_store(uint32_t nj, P1Rows& R) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t q = lane / 6u, c = lane % 6u;
+  for (uint32_t j = q < 5u ? q : nj; j < nj; j += 5) {
+    const uint4 what = row_chunk(R, j, 2);
+    const uint4 vb = row_chunk(R, j, 1);
+    if (!((what.x >> c) & 1u)) continue;
+    const uint32_t s = (what.x >> 8) & 7u, timers = kTimers ? what.x >> 16 : 0u;
+    const uint32_t w = c < 4u ? reinterpret_cast<const uint32_t*>(&row_chunk(R, j, 0))[c] : (c == 4u ? vb.x : vb.y);
+    const uint32_t off = c < 4u ? key_off(timers, s) + 4u * c : value_off(timers, s) + 4u * (c - 4u);
+    *reinterpret_cast<uint32_t*>(hi64(vb) + off) = w;
+  }
+  const uint32_t half = lane & 1u;
+  for (uint32_t j = lane >> 1; j < nj; j += 16) {
+    const uint4 what = row_chunk(R, j, 2);
+    if (!((what.x >> (6u + half)) & 1u)) continue;
+    const uint32_t off = 2u * ((what.x >> 8) & 7u) + (half ? kExpiryOff : 0u);
+    *reinterpret_cast<uint16_t*>(hi64(row_chunk(R, j, 1)) + off) = (uint16_t)(half ? what.y >> 16 : what.y);
+  }
+}
+
+// The lists a thread appends to in phase 1: displacement passes, followers, sticky.
+using P1Lists = BlockLists<3>;
+
+// One key of phase 1 (every thread of the block calls this; act: it has a
+// key). A warp takes the steps of all its keys together, so its lanes' memory
+// round trips overlap: the key; the set's CAS and the primary's header; the
+// secondary's header, for the keys whose filter bits are set or whose primary
+// has no room; the claim; the entry; the publication.
+template <bool kTimers>
+__device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __restrict__ keys,
+                                           const uint64_t* __restrict__ vals, uint32_t now, uint32_t expiry,
+                                           uint8_t* __restrict__ status, const Workspace& ws, uint64_t i64, bool act,
+                                           P1Rows& R, P1Lists& lists) {
+  const uint32_t i = (uint32_t)i64;
+  if (act && !ts.valid(i)) {
+    status[i] = kStNoTable;
+    act = false;
+  }
+  TableView t{};
+  uint32_t tid = 0, owner = i;
+  Key k{0, 0};
+  uint64_t v = 0, h1 = 0;
+  Addr a{};
+  SetProbe probe{};
+  if (act) {
+    tid = ts.id(i);
+    t = ts.of(i);
+    k = load_key(keys, i);
+    v = vals[i];
+    a = address_of(k, t.nb, t.seed, h1);
+    probe = set_probe(ws, h1, tid, i);
+  }
+  const bool timers = kTimers && t.timers;
+  Snap s;
+  p1_fetch<kTimers>(t, a.b1, act, R, s);
+  if (act) owner = set_owner(ws, ts, keys, k, tid, i, probe);
+  const bool mine = act && owner == i;
+  P1Bucket r{}, r2{};
+  bool maybe2 = false, have2 = false;
+  if (mine) {
+    r = p1_bucket(t, a.b1, s, a.tag, timers, now);
+    maybe2 = (r.bloom & a.bits) == a.bits;  // the filter allows the secondary
+    have2 = maybe2 || !claimable(r.ctrl, r.dead);
+  }
+  p1_fetch<kTimers>(t, a.b2, have2, R, s);
+  uint8_t st = 0;
+  P1Work work = kP1None;
+  uint32_t flip = 0;  // publication: the bits of the ctrl word to flip
+  int sl = -1;
+  bool sticky = false;
+  if (mine) {
+    if ((sl = p1_find(t, r, k)) >= 0) st = p1_stored(t, r, (uint32_t)sl, timers, work);
+    if (have2) r2 = p1_bucket(t, a.b2, s, a.tag, timers, now);
+    if (!st && maybe2 && (sl = p1_find(t, r2, k)) >= 0) {
+      st = p1_stored(t, r2, (uint32_t)sl, timers, work);
+      if (st) r = r2;
+    }
+    if (!st) {
+      if (!claimable(r.ctrl, r.dead)) r = r2;
+      for (;;) {
+        uint32_t prev = 0;
+        sl = claim_slot(t, r, prev);
+        if (sl >= 0) {
+          work = kP1Place;
+          st = kStInserted;
+          flip = 1u << sl;
+          sticky = kTimers && ((prev >> sl) & 1u);  // held a dead entry
+          if (!sticky) flip |= claim_bit(sl);
+          if (sticky && ((prev >> (kInsecShift + sl)) & 1u)) evict_displaced(t, tid, r.b, sl, ws);
+          if (r.b == a.b2) {  // Sec. 4.1: displaced to the secondary
+            flip |= 1u << (kInsecShift + sl);
+            atomicOr(reinterpret_cast<unsigned long long*>(bloom_ptr(t, a.b1)), (unsigned long long)a.bits);
+            atomicAdd(moved_ptr(t, a.b1), 1u);
+          }
+          break;
+        }
+        if (sl == -2) {
+          st = kStBusy;
+          latch_error(t, kErrLockTimeout);
+          break;
+        }
+        if (r.b == a.b2) break;
+        // the primary filled up under the claim: its secondary
+        if (!have2) {
+          p1_fetch_one(t, a.b2, timers, s);
+          r2 = p1_bucket(t, a.b2, s, a.tag, timers, now);
+        }
+        r = r2;
+      }
+    }
+    if (st) status[i] = st;
+  }
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t jobs = __ballot_sync(kWarpAll, work != kP1None);
+  if (work != kP1None) {
+    const uint32_t j = __popc(jobs & ((1u << lane) - 1u));
+    const unsigned long long bp = reinterpret_cast<unsigned long long>(bucket_ptr(t, r.b));
+    const uint32_t words = (work == kP1Place ? 0x7Fu : 0x30u) | (timers ? 0x80u : 0u);
+    row_chunk(R, j, 0) = make_uint4((uint32_t)k.k0, (uint32_t)(k.k0 >> 32), (uint32_t)k.k1, (uint32_t)(k.k1 >> 32));
+    row_chunk(R, j, 1) = make_uint4((uint32_t)v, (uint32_t)(v >> 32), (uint32_t)bp, (uint32_t)(bp >> 32));
+    row_chunk(R, j, 2) =
+        make_uint4(words | (uint32_t)sl << 8 | (timers ? 0x10000u : 0u), (a.tag & 0xFFFFu) | expiry << 16, 0u, 0u);
+  }
+  __syncwarp();
+  p1_store<kTimers>(__popc(jobs), R);
+  fence_acq_rel();  // every lane's stores before any busy bit
+  __syncwarp();
+  if (work == kP1Place) atomicXor(ctrl_ptr(t, r.b), flip);
+  sticky |= work == kP1Revive;
+  const bool queued = mine && !st, follows = act && !mine;
+  uint32_t at[3];
+  lists_append<3>(lists, {ws.counters + kCntPending, ws.counters + kCntFollowers, ws.counters + kCntSticky},
+                  {queued, follows, sticky}, at);
+  if (queued) ws.pending[at[0]] = i;
+  if (follows) write_follower(ws, at[1], i, owner);
+  if (sticky) ws.sticky[at[2]] = (unsigned long long)i << 32 | r.b;
+}
+
+template <bool kTimers>
+__global__ void __launch_bounds__(kThreads, 4) insert_phase1(TableSet ts, const uint8_t* __restrict__ keys,
+                                                             const uint64_t* __restrict__ vals, uint64_t n,
+                                                             uint32_t now, uint32_t expiry,
+                                                             uint8_t* __restrict__ status, Workspace ws) {
+  __shared__ P1Rows rows[kThreads / 32];
+  __shared__ P1Lists lists;
+  lists_init(lists);
   pdl_wait();
   pdl_release();
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i < n) phase1_one(ts, keys, vals, now, expiry, status, ws, i);
-}
-
-// Publication of phase 1's claims: each claimed slot's claimed bit is cleared
-// and its busy (and in_secondary) bits set, in one atomic XOR per key. From
-// here on the new entries are visible to every search.
-__device__ __forceinline__ void publish_one(const TableSet& ts, const Workspace& ws, uint64_t i) {
-  const unsigned long long r = ws.claim[i];
-  if (!r) return;
-  const TableView t = ts.of(i);
-  atomicXor(ctrl_ptr(t, (uint32_t)(r >> 32)), (uint32_t)r);
-}
-
-__global__ void __launch_bounds__(kThreads) insert_publish(TableSet ts, uint64_t n, Workspace ws) {
-  pdl_wait();
-  pdl_release();
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i < n) publish_one(ts, ws, i);
+  const uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x;
+  phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
 }
 
 // --------------------------------------------------------------- phase 2
@@ -478,8 +544,6 @@ __device__ int bfs(const TableView& t, const Addr& a, uint32_t now, const Queue&
 // in queue order with a free or dead slot, a shortest path as in the thread
 // form. q: the warp's queue (kBfsNodes nodes); seen: its set. Every lane
 // returns the same node index (or -1) and hole.
-constexpr uint32_t kWarpAll = 0xFFFFFFFFu;
-
 template <int kBfsNodes>
 struct WarpSeen {
   // smallest power of two at least 1.5 x (kBfsNodes + the 256 children of a round)
@@ -778,7 +842,7 @@ __device__ void move1_range(const TableSet& ts, const uint8_t* __restrict__ keys
   for (uint32_t j = worker; j < count; j += workers) {
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
-    const uint64_t v = value_of(ws, vals, i);
+    const uint64_t v = vals[i];
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
     uint32_t x = 0, sx = 0, y = 0, hole = 0;
@@ -841,6 +905,7 @@ __global__ void __launch_bounds__(kThreads) insert_move1(TableSet ts, const uint
                                                          uint32_t* next, uint32_t* next_count) {
   pdl_wait();
   pdl_release();
+  follower_ranges(ws, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
   move1_range(ts, keys, vals, now, expiry, status, ws, list, count_ptr, next, next_count,
               blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
@@ -862,7 +927,7 @@ __device__ void phase2_range(const TableSet& ts, const uint8_t* __restrict__ key
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
     const uint32_t tid = ts.id(i);
-    const uint64_t v = value_of(ws, vals, i);
+    const uint64_t v = vals[i];
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
     uint8_t st = kStFull;
@@ -908,7 +973,7 @@ __device__ void phase2_range_warp(const TableSet& ts, const uint8_t* __restrict_
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
     const uint32_t tid = ts.id(i);
-    const uint64_t v = value_of(ws, vals, i);
+    const uint64_t v = vals[i];
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
     uint8_t st = kStFull;
@@ -998,21 +1063,24 @@ __global__ void __launch_bounds__(kThreadsPerBlock) insert_phase2(TableSet ts, c
 }
 
 // ----------------------------------------------------- fixup and finish
-// The two parts touch disjoint words (filters of the fixup list's buckets;
-// status bytes of non-leader keys), so one launch runs both: every thread
-// takes its share of the fixup list, and thread i < n finishes key i.
-__device__ void fixup_finish_range(const TableSet& ts, uint64_t n, uint8_t* __restrict__ status, const Workspace& ws,
-                                   uint64_t worker, uint64_t workers) {
+// What is left after the last pass, each part a list that is usually short or
+// empty: the deferred filter resets, the claimed bits that phase 1 left set in
+// timers tables, and the followers (dedup.cuh). The parts touch disjoint words,
+// so one launch runs them: filters of buckets whose moved counter is zero; ctrl
+// words; the status bytes and stored values of groups with followers.
+__device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict__ keys,
+                                   const uint64_t* __restrict__ vals, uint8_t* __restrict__ status,
+                                   const Workspace& ws, uint64_t worker, uint64_t workers) {
   const uint64_t stride = workers;
   const uint64_t i = worker;
-  if (ld32_cg(ws.counters + 2)) {  // the list overflowed: scan every bucket of every table
+  if (ld32_cg(ws.counters + kCntFixupOverflow)) {  // the list overflowed: scan every bucket of every table
     for (uint32_t tb = 0; tb < ts.n_tables; ++tb) {
       const TableView t = ts.table(tb);
       for (uint64_t b = i; b < t.nb; b += stride)
         if (ld32_cg(moved_ptr(t, (uint32_t)b)) == 0u) st64_cg(bloom_ptr(t, (uint32_t)b), 0ull);
     }
   } else {
-    const uint32_t count = min(ld32_cg(ws.counters + 1), ws.fix_cap);
+    const uint32_t count = min(ld32_cg(ws.counters + kCntFixup), ws.fix_cap);
     for (uint64_t j = i; j < count; j += stride) {
       const unsigned long long e = ws.fixup[j];
       const TableView t = ts.table((uint32_t)(e >> 32));
@@ -1020,28 +1088,62 @@ __device__ void fixup_finish_range(const TableSet& ts, uint64_t n, uint8_t* __re
       if (ld32_cg(moved_ptr(t, b)) == 0u) st64_cg(bloom_ptr(t, b), 0ull);
     }
   }
-  for (uint64_t j = i; j < n; j += stride) {
-    if (status[j] != kStFollower) continue;  // a leader: its outcome is final
-    const uint32_t leader = ld32_cg(ws.first_at(ws.slot_of[j]));
-    const uint8_t st = status[leader];
-    status[j] = (st == kStInserted || st == kStUpdated) ? kStUpdated : st;  // FULL, BUSY, NO_TABLE copy through
+  const uint32_t sticky = ld32_cg(ws.counters + kCntSticky);
+  for (uint64_t j = i; j < sticky; j += stride) {
+    const unsigned long long e = ws.sticky[j];
+    atomicAnd(ctrl_ptr(ts.of(e >> 32), (uint32_t)e), ~(kBusyMask << kClaimShift));
+  }
+  const uint32_t followers = ld32_cg(ws.counters + kCntFollowers);
+  for (uint64_t j = i; j < followers; j += stride) {
+    const uint2 f = ws.followers[j];
+    const uint2 range = ws.range[f.y];
+    const bool last = f.x == range.y;  // its value is the one that stays
+    // the buckets of a last occurrence are requested before the owner's outcome is looked at
+    TableView t{};
+    Key k{0, 0};
+    Addr a{};
+    Snap s1{}, s2{};
+    if (last) {
+      t = ts.of(f.x);
+      k = load_key(keys, f.x);
+      a = address_of(k, t.nb, t.seed);
+      ld256_cg(bucket_ptr(t, a.b1), s1.w);
+      ld256_cg(bucket_ptr(t, a.b2), s2.w);
+    }
+    // the owner's outcome; the group's lowest index takes it over (from INSERTED the owner then
+    // becomes UPDATED, which every other follower reports for either)
+    uint8_t st = *reinterpret_cast<volatile uint8_t*>(status + f.y);
+    const bool stored = st == kStInserted || st == kStUpdated;
+    if (st == kStInserted && f.x == range.x) {
+      status[f.y] = kStUpdated;
+    } else if (stored) {
+      st = kStUpdated;  // FULL and BUSY copy through
+    }
+    status[f.x] = st;
+    if (last && stored) {
+      const int in1 = find_key(t, a.b1, (uint32_t)s1.w[3], s1, k, a.tag);
+      const int in2 = in1 >= 0 ? -1 : find_key(t, a.b2, (uint32_t)s2.w[3], s2, k, a.tag);
+      if (in1 >= 0) st64_cg(value_ptr(t, a.b1, in1), vals[f.x]);
+      if (in2 >= 0) st64_cg(value_ptr(t, a.b2, in2), vals[f.x]);
+    }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) insert_fixup_finish(TableSet ts, uint64_t n, uint8_t* __restrict__ status,
-                                                                Workspace ws) {
+__global__ void __launch_bounds__(kThreads) insert_fixup_finish(TableSet ts, const uint8_t* __restrict__ keys,
+                                                                const uint64_t* __restrict__ vals,
+                                                                uint8_t* __restrict__ status, Workspace ws) {
   pdl_wait();
   pdl_release();
-  fixup_finish_range(ts, n, status, ws, blockIdx.x * (uint64_t)blockDim.x + threadIdx.x,
+  fixup_finish_range(ts, keys, vals, status, ws, blockIdx.x * (uint64_t)blockDim.x + threadIdx.x,
                      (uint64_t)gridDim.x * blockDim.x);
 }
 
 // --------------------------------------------------- single-launch insert
 // The whole insert call of a small batch in one cooperative launch: the
-// stages of the chain above (dedup, phase 1, publication, the one-move pass,
-// the three search passes, fixup and finish) run in order, separated by a
+// stages of the chain above (phase 1, the one-move pass, the three search
+// passes, fixup and finish) run in order, separated by a
 // grid barrier instead of kernel boundaries. A small batch spends most of a
-// chain's time in the chain's nine dependent launches (each one's start and
+// chain's time in the chain's seven dependent launches (each one's start and
 // drain); here it pays two (the workspace clear and this kernel). All blocks
 // are resident at once (cooperative launch, grid sized by the occupancy the
 // kernel reaches), so the barrier cannot wait on a block that has not
@@ -1057,6 +1159,7 @@ constexpr unsigned kSingleMinBlocks = 8;
 // the bounded lock waits a stage may contain, so a barrier gives up only if a block never arrives.
 constexpr int kBarrierSpins = 1 << 22;
 
+static_assert((kSingleThreads / 32) * sizeof(P1Rows) <= kSingleSmem, "phase 1 rows exceed the shared memory");
 static_assert(96 * 64 * sizeof(Node) <= kSingleSmem, "grid pass queues exceed the shared memory");
 static_assert((kSingleThreads / 32) * warp_search_bytes<96>() <= kSingleSmem,
               "grid pass state (one warp per key) exceeds the shared memory");
@@ -1105,159 +1208,89 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
                                                                          const uint64_t* __restrict__ vals, uint64_t n,
                                                                          uint32_t now, uint32_t expiry,
                                                                          uint8_t* __restrict__ status, Workspace ws) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint32_t* bar_count = ws.counters + 8;
-  uint32_t* bar_gen = ws.counters + 9;
+  extern __shared__ __align__(128) uint8_t smem[];
+  uint32_t* bar_count = ws.counters + kCntBarrier;
+  uint32_t* bar_gen = ws.counters + kCntBarrier + 1;
   const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
   bool ok = true;
-  for (uint64_t i = tid; i < n; i += threads) dedup_one(keys, ts, ws, i);
+  P1Rows* rows = reinterpret_cast<P1Rows*>(smem);
+  __shared__ P1Lists lists;
+  lists_init(lists);
+  for (uint64_t first = blockIdx.x * (uint64_t)kSingleThreads; first < n; first += threads) {  // whole blocks
+    const uint64_t i = first + threadIdx.x;
+    phase1_one<true>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
+  }
   ok &= grid_barrier(bar_count, bar_gen);
-  for (uint64_t i = tid; i < n; i += threads) phase1_one(ts, keys, vals, now, expiry, status, ws, i);
-  ok &= grid_barrier(bar_count, bar_gen);
-  for (uint64_t i = tid; i < n; i += threads) publish_one(ts, ws, i);
-  ok &= grid_barrier(bar_count, bar_gen);
+  if (ld32_cg(ws.counters + kCntFollowers)) {
+    follower_ranges(ws, (uint32_t)tid, (uint32_t)threads);
+    if (!ld32_cg(ws.counters + kCntPending)) ok &= grid_barrier(bar_count, bar_gen);
+  }
   // lists as in the chain: pending [0] -> one move -> retry [3] -> grid search -> pending [5] ->
   // second pass -> retry [6] -> last pass. A pass whose list is empty is skipped with its barrier;
   // every block reads the same count (final before the barrier), so all skip alike.
-  if (ld32_cg(ws.counters + 0)) {
-    move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, ws.counters + 0, ws.retry, ws.counters + 3,
+  if (ld32_cg(ws.counters + kCntPending)) {
+    move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, ws.counters + kCntPending, ws.retry, ws.counters + kCntMoved1,
                 (uint32_t)tid, (uint32_t)threads);
     ok &= grid_barrier(bar_count, bar_gen);
   }
   Node* nodes = reinterpret_cast<Node*>(smem);
   const uint32_t w = threadIdx.x >> 5;
-  if (const uint32_t listed = ld32_cg(ws.counters + 3)) {
+  if (const uint32_t listed = ld32_cg(ws.counters + kCntMoved1)) {
     if (listed <= kGridWarpKeys) {  // a short list: one warp per key
       uint8_t* mine = smem + w * warp_search_bytes<96>();
       phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                               ws.counters + 5, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
+                               ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
                                reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)),
                                blockIdx.x * (kSingleThreads / 32) + w, gridDim.x * (kSingleThreads / 32));
     } else if (threadIdx.x < 64) {
       const Queue q{nodes + threadIdx.x, 64};
       phase2_range<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                          ws.counters + 5, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
+                          ws.counters + kCntGrid, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
     }
     ok &= grid_barrier(bar_count, bar_gen);
   }
-  if (ld32_cg(ws.counters + 5)) {
+  if (ld32_cg(ws.counters + kCntGrid)) {
     constexpr size_t kPer = warp_search_bytes<192>();
     uint8_t* mine = smem + w * kPer;
-    phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, ld32_cg(ws.counters + 5), ws.retry,
-                              ws.counters + 6, kSecondPassKeys, reinterpret_cast<Node*>(mine),
+    phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, ld32_cg(ws.counters + kCntGrid), ws.retry,
+                              ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
                               reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)),
                               blockIdx.x * (kSingleThreads / 32) + w, gridDim.x * (kSingleThreads / 32));
     ok &= grid_barrier(bar_count, bar_gen);
   }
-  if (ld32_cg(ws.counters + 6)) {
+  if (ld32_cg(ws.counters + kCntSecond)) {
     if (w == 0)
-      phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, ld32_cg(ws.counters + 6),
+      phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, ld32_cg(ws.counters + kCntSecond),
                                  (uint32_t*)nullptr, (uint32_t*)nullptr, kLastPassKeys, nodes,
                                  reinterpret_cast<uint32_t*>(smem + 2048 * sizeof(Node)), blockIdx.x, gridDim.x);
     ok &= grid_barrier(bar_count, bar_gen);
   }
-  fixup_finish_range(ts, n, status, ws, tid, threads);
+  fixup_finish_range(ts, keys, vals, status, ws, tid, threads);
   if (!ok && threadIdx.x == 0) latch_error(ts.table(0), kErrLockTimeout);
 }
 
 // ------------------------------------------------------- workspace reset
-// The set's words alternate first (empty) and last (0), so each 16-byte
-// vector holds two positions.
-__global__ void __launch_bounds__(kThreads) workspace_clear(uint32_t* __restrict__ counters, uint32_t counter_words,
-                                                            uint4* __restrict__ set, uint64_t n_vec,
-                                                            uint4* __restrict__ dup, uint64_t dup_vec) {
+__global__ void __launch_bounds__(kThreads) workspace_clear(uint32_t* __restrict__ counters,
+                                                            uint4* __restrict__ set, uint64_t n_vec) {
   pdl_release();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (tid < counter_words) counters[tid] = 0u;
-  for (uint64_t j = tid; j < n_vec; j += stride) set[j] = make_uint4(kEmpty, 0u, kEmpty, 0u);
-  for (uint64_t j = tid; j < dup_vec; j += stride) dup[j] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-__global__ void __launch_bounds__(kThreads) delete_kernel(TableSet ts, const uint8_t* __restrict__ keys, uint64_t n,
-                                                          uint32_t now, uint8_t* __restrict__ status, Workspace ws) {
-  pdl_wait();
-  pdl_release();
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (!ts.valid(i)) {
-    status[i] = kStNoTable;
-    return;
-  }
-  uint32_t last;
-  if (!is_leader(ws, i, last)) {
-    status[i] = kStNotFound;
-    return;
-  }
-  const TableView t = ts.of(i);
-  const Key k = load_key(keys, i);
-  const Addr a = address_of(k, t.nb, t.seed);
-  uint64_t h[4];
-  ld256_cg(bucket_ptr(t, a.b1), h);
-  uint32_t b = a.b1;
-  Snap s;
-  s.w[0] = h[0];
-  s.w[1] = h[1];
-  int slot = find_key(t, b, (uint32_t)h[3], s, k, a.tag);
-  if (slot < 0 && (h[2] & a.bits) == a.bits) {
-    b = a.b2;
-    ld256_cg(bucket_ptr(t, b), s.w);
-    slot = find_key(t, b, (uint32_t)s.w[3], s, k, a.tag);
-  }
-  uint8_t st = kStNotFound;
-  if (slot >= 0) {
-    const bool was_alive = !t.timers || alive16(ld16_cg(expiry_ptr(t, b, slot)), now);
-    const uint32_t old = atomicAnd(ctrl_ptr(t, b), ~((1u << slot) | (1u << (kInsecShift + slot))));
-    // Sec. 4.1: removing a displaced key decrements its primary's counter; at
-    // zero the filter is reset. No filter bit is set during a delete batch.
-    if ((old >> (kInsecShift + slot)) & 1u) {
-      if (atomicSub(moved_ptr(t, a.b1), 1u) == 1u)
-        atomicExch(reinterpret_cast<unsigned long long*>(bloom_ptr(t, a.b1)), 0ull);
-    }
-    st = was_alive ? kStDeleted : kStNotFound;
-  }
-  status[i] = st;
-}
-
-unsigned grid_for(uint64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
-
-// Launch a kernel of an insert or delete call after its predecessor on the
-// same stream, with programmatic stream serialization (see pdl_wait).
-template <typename... Params, typename... Args>
-cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned block, cudaStream_t s, Args... args) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (tid < kCounterWords) counters[tid] = 0u;
+  for (uint64_t j = tid; j < n_vec; j += stride) set[j] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
 }
 
 }  // namespace
 
-cudaError_t launch_workspace_clear(const Workspace& ws, uint32_t counter_words, uint64_t n, cudaStream_t s) {
-  // m is a power of two >= 64 and the set is 256-byte aligned: 2m words clear
-  // as m / 2 whole 16-byte vectors; dup (256-byte aligned, its part of the
-  // layout rounded up to 256 bytes) clears as ceil(n / 16) vectors
-  const uint64_t n_vec = ((uint64_t)ws.m_mask + 1) / 2;
-  const uint64_t dup_vec = (n + 15) / 16;
-  uint64_t want = n_vec > counter_words ? n_vec : counter_words;
-  want = want > dup_vec ? want : dup_vec;
+cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s) {
+  // m is a power of two >= 64 and the set is 256-byte aligned: whole 16-byte vectors
+  const uint64_t n_vec = ((uint64_t)ws.m_mask + 1) / 4;
+  const uint64_t want = n_vec > kCounterWords ? n_vec : kCounterWords;
   const uint64_t blocks = (want + kThreads - 1) / kThreads;
   const uint64_t cap = 16ull * device_sm_count();
   workspace_clear<<<(unsigned)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(
-      ws.counters, counter_words, reinterpret_cast<uint4*>(ws.set), n_vec, reinterpret_cast<uint4*>(ws.dup), dup_vec);
+      ws.counters, reinterpret_cast<uint4*>(ws.set), n_vec);
   return cudaGetLastError();
-}
-
-cudaError_t launch_dedup(const TableSet& ts, const uint8_t* keys, uint64_t n, const Workspace& ws, cudaStream_t s) {
-  return launch_chained(dedup_kernel, grid_for(n, kThreads), kThreads, s, keys, n, ts, ws);
 }
 
 namespace {
@@ -1322,42 +1355,38 @@ cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_
     const int per_sm = single_launch_blocks_per_sm();
     if (per_sm > 0) return launch_single(ts, keys, vals, n, now, expiry, status, ws, s, per_sm);
   }
-  cudaError_t e = launch_dedup(ts, keys, n, ws, s);
-  if (e != cudaSuccess) return e;
-  e = launch_chained(insert_phase1, grid_for(n, kThreads), kThreads, s, ts, keys, vals, n, now, expiry, status, ws);
-  if (e != cudaSuccess) return e;
-  e = launch_chained(insert_publish, grid_for(n, kThreads), kThreads, s, ts, n, ws);
+  const unsigned sms = (unsigned)device_sm_count();
+  cudaError_t e;
+  e = launch_chained(ts.any_timers ? insert_phase1<true> : insert_phase1<false>, grid_for(n, kThreads), kThreads, s, ts,
+                     keys, vals, n, now, expiry, status, ws);
   if (e != cudaSuccess) return e;
   // lists: phase 1 -> pending [0] -> move1 -> retry [3] -> grid search ->
   // pending [5] -> second search -> retry [6] -> last search
-  const unsigned sms = (unsigned)device_sm_count();
-  e = launch_chained(insert_move1, sms * 16, kThreads, s, ts, keys, vals, now, expiry, status, ws,
-                     (const uint32_t*)ws.pending, (const uint32_t*)(ws.counters + 0), ws.retry, ws.counters + 3);
+  // each pass's list holds at most n keys: no more blocks than that many keys can use
+  const auto cap = [n](unsigned blocks, unsigned keys_per_block) {
+    const uint64_t want = (n + keys_per_block - 1) / keys_per_block;
+    return want < blocks ? (unsigned)want : blocks;
+  };
+  e = launch_chained(insert_move1, cap(sms * 16, kThreads), kThreads, s, ts, keys, vals, now, expiry, status, ws,
+                     (const uint32_t*)ws.pending, (const uint32_t*)(ws.counters + kCntPending), ws.retry, ws.counters + kCntMoved1);
   if (e != cudaSuccess) return e;
-  e = launch_chained(insert_phase2<kP2Threads, 96, 4>, sms * 4, kP2Threads, s, ts, keys, vals, now, expiry, status,
-                     ws, (const uint32_t*)ws.retry, (const uint32_t*)(ws.counters + 3), ws.pending, ws.counters + 5,
+  e = launch_chained(insert_phase2<kP2Threads, 96, 4>, cap(sms * 4, kP2Threads / 32), kP2Threads, s, ts, keys, vals, now, expiry, status,
+                     ws, (const uint32_t*)ws.retry, (const uint32_t*)(ws.counters + kCntMoved1), ws.pending, ws.counters + kCntGrid,
                      0xFFFFFFFFu);
   if (e != cudaSuccess) return e;
   // second pass, one warp per key: the keys the grid pass could not place
-  e = launch_chained(insert_phase2_warp<8, 192, 5>, sms * 2, 8 * 32, s, ts, keys, vals, now, expiry, status, ws,
-                     (const uint32_t*)ws.pending, (const uint32_t*)(ws.counters + 5), ws.retry, ws.counters + 6,
+  e = launch_chained(insert_phase2_warp<8, 192, 5>, cap(sms * 2, 8), 8 * 32, s, ts, keys, vals, now, expiry, status, ws,
+                     (const uint32_t*)ws.pending, (const uint32_t*)(ws.counters + kCntGrid), ws.retry, ws.counters + kCntSecond,
                      kSecondPassKeys);
   if (e != cudaSuccess) return e;
   // last pass, one warp per key: the widest search; a key is FULL only if it finds no path
-  e = launch_chained(insert_phase2_warp<1, 2048, 6>, kLastPassKeys, 32, s, ts, keys, vals, now, expiry, status, ws,
-                     (const uint32_t*)ws.retry, (const uint32_t*)(ws.counters + 6), (uint32_t*)nullptr,
+  e = launch_chained(insert_phase2_warp<1, 2048, 6>, cap(kLastPassKeys, 1), 32, s, ts, keys, vals, now, expiry, status, ws,
+                     (const uint32_t*)ws.retry, (const uint32_t*)(ws.counters + kCntSecond), (uint32_t*)nullptr,
                      (uint32_t*)nullptr, kLastPassKeys);
   if (e != cudaSuccess) return e;
   const unsigned fin_blocks = grid_for(n, kThreads);
-  return launch_chained(insert_fixup_finish, fin_blocks > sms * 2 ? fin_blocks : sms * 2, kThreads, s, ts, n, status,
-                        ws);
-}
-
-cudaError_t launch_delete(const TableSet& ts, const uint8_t* keys, uint64_t n, uint32_t now, uint8_t* status,
-                          const Workspace& ws, cudaStream_t s) {
-  cudaError_t e = launch_dedup(ts, keys, n, ws, s);
-  if (e != cudaSuccess) return e;
-  return launch_chained(delete_kernel, grid_for(n, kThreads), kThreads, s, ts, keys, n, now, status, ws);
+  return launch_chained(insert_fixup_finish, fin_blocks < sms * 2 ? fin_blocks : sms * 2, kThreads, s, ts, keys, vals,
+                        status, ws);
 }
 
 }  // namespace ckpp

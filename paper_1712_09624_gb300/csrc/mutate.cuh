@@ -5,10 +5,11 @@
 // Concurrency rules of the insert kernels (one table, one batch at a time):
 //  * phase 1 takes no lock: a key claims a free or dead slot with a CAS on the
 //    bucket's ctrl word (claimed bits 16-23), writes its entry into the
-//    claimed slot, and the next kernel publishes the claim (claimed -> busy);
-//    searches look at busy slots only, so a claimed slot is invisible until
-//    then. In-place updates touch live entries, which no claim can take;
-//  * in the displacement passes (after publication) a bucket's busy /
+//    claimed slot, and publishes it behind a fence (claimed -> busy); searches
+//    look at busy slots only, so a claimed slot is invisible until then, and
+//    read the key of a matching slot behind a fence of their own. In-place
+//    updates touch live entries, which no claim can take;
+//  * in the displacement passes a bucket's busy /
 //    in_secondary bits, tags, expiries, keys and values change only while its
 //    lock bit (ctrl bit 31) is held; the new ctrl word is published by the
 //    unlocking exchange;
@@ -219,25 +220,29 @@ __device__ __forceinline__ int find_key(const TableView& t, uint32_t b, uint32_t
 }
 
 __device__ __forceinline__ void push_fixup(const Workspace& ws, uint32_t table, uint32_t b) {
-  const uint32_t idx = atomicAdd(ws.counters + 1, 1u);
+  const uint32_t idx = atomicAdd(ws.counters + kCntFixup, 1u);
   if (idx < ws.fix_cap) {
     ws.fixup[idx] = ((unsigned long long)table << 32) | b;
   } else {
-    atomicExch(ws.counters + 2, 1u);
+    atomicExch(ws.counters + kCntFixupOverflow, 1u);
   }
 }
 
-// Remove the (dead) entry in slot s of locked bucket b of table tid: if it sits in its
-// secondary bucket its primary's moved counter is decremented (Sec. 4.1).
+// Upkeep for a dead entry that sits in its secondary bucket b, slot s, and is
+// about to be overwritten: its primary's moved counter drops (Sec. 4.1); a
+// counter that reaches zero is queued for the filter reset of the finishing pass.
+__device__ __forceinline__ void evict_displaced(const TableView& t, uint32_t tid, uint32_t b, uint32_t s,
+                                                const Workspace& ws) {
+  Key k;
+  ld128_cg(key_ptr(t, b, s), k.k0, k.k1);
+  const Addr a = address_of(k, t.nb, t.seed);
+  if (atomicSub(moved_ptr(t, a.b1), 1u) == 1u) push_fixup(ws, tid, a.b1);
+}
+
+// Remove the (dead) entry in slot s of locked bucket b of table tid.
 __device__ __forceinline__ void evict_entry(const TableView& t, uint32_t tid, uint32_t b, uint32_t s, uint32_t& ctrl,
                                             const Workspace& ws) {
-  if ((ctrl >> (kInsecShift + s)) & 1u) {
-    Key k;
-    ld128_cg(key_ptr(t, b, s), k.k0, k.k1);
-    const Addr a = address_of(k, t.nb, t.seed);
-    const uint32_t old = atomicSub(moved_ptr(t, a.b1), 1u);
-    if (old == 1u) push_fixup(ws, tid, a.b1);
-  }
+  if ((ctrl >> (kInsecShift + s)) & 1u) evict_displaced(t, tid, b, s, ws);
   ctrl &= ~((1u << s) | (1u << (kInsecShift + s)));
 }
 

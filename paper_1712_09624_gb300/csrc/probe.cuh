@@ -37,6 +37,7 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 // Whether the keys' tables have timers: known for the whole launch (a plain
 // lookup is over one table) or per key (the batched form).
 enum TimersMode : int { kNoTimers = 0, kWithTimers = 1, kTimersPerKey = 2 };
+constexpr uint32_t kNoSlot = 0xFFu;
 constexpr uint32_t kDone = 4;  // stages: 0 b1 line 0, 1 b1 line 1, 2 b2 line 0, 3 b2 line 1, 4 done
 
 // One key's lookup, owned by one lane.
@@ -52,13 +53,13 @@ struct Probe {
   bool skip;        // pessimistic: the key is resolved; the read is made for its cost only
   bool found;
   uint64_t value;
-  uint32_t hb, hs;  // bucket and slot of the hit (for a refresh)
+  uint32_t hb, hs;  // bucket and slot of the key's entry, alive (found) or dead; kNoSlot: not stored
   uint32_t nsec, nrec, nline1;  // counting mode
 };
 
 __device__ __forceinline__ void probe_init(Probe& p, const Key& k, const uint8_t* buckets, uint64_t nb, uint64_t seed,
-                                           uint32_t timers) {
-  const uint64_t h1 = hash_key(k, seed);
+                                           uint32_t timers, uint64_t& h1) {
+  h1 = hash_key(k, seed);
   const uint64_t h2 = hash_key(k, seed ^ kSeed2Xor);
   p.k = k;
   p.buckets = buckets;
@@ -74,8 +75,15 @@ __device__ __forceinline__ void probe_init(Probe& p, const Key& k, const uint8_t
   p.skip = false;
   p.found = false;
   p.value = 0;
-  p.hb = p.hs = 0;
+  p.hb = 0;
+  p.hs = kNoSlot;
   p.nsec = p.nrec = p.nline1 = 0;
+}
+
+__device__ __forceinline__ void probe_init(Probe& p, const Key& k, const uint8_t* buckets, uint64_t nb, uint64_t seed,
+                                           uint32_t timers) {
+  uint64_t h1;
+  probe_init(p, k, buckets, nb, seed, timers, h1);
 }
 
 // Shared-memory slab of one warp: the line jobs of an iteration, posted by
@@ -90,8 +98,6 @@ struct WarpStage {
 
 __device__ __forceinline__ uint4 lds128(const uint8_t* p) { return *reinterpret_cast<const uint4*>(p); }
 __device__ __forceinline__ uint64_t lds64(const uint8_t* p) { return *reinterpret_cast<const uint64_t*>(p); }
-__device__ __forceinline__ uint64_t lo64(const uint4& v) { return (uint64_t)v.x | (uint64_t)v.y << 32; }
-__device__ __forceinline__ uint64_t hi64(const uint4& v) { return (uint64_t)v.z | (uint64_t)v.w << 32; }
 
 // Mask of the 8 tags (16-bit lanes of tg) equal to tag: per 32-bit word, a
 // 16-bit lane of x = word ^ (tag, tag) is zero exactly when the top bit of
@@ -182,7 +188,7 @@ __device__ __forceinline__ void examine(Probe& p, const uint8_t* L, uint32_t sw,
     p.stage = 2;
     p.carry = 0;
   } else {
-    resolve<kVariant>(p, false, 0, b, 0);
+    resolve<kVariant>(p, false, 0, b, kNoSlot);
   }
 }
 
