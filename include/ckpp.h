@@ -279,16 +279,14 @@ int ckpp_bulk_insert(ckpp_table* table, const ckpp_key* keys, const uint64_t* va
  *                              duplicate resolution and the slot claims, the
  *                              one-move pass, three cuckoo-path searches, the
  *                              filter fixup, each launched to start while its
- *                              predecessor drains;
+ *                              predecessor drains; a batch of at most 2048
+ *                              keys runs the same stages in one launch of one
+ *                              thread-block cluster;
  *   CKPP_INSERT_LAUNCH_SINGLE  one cooperative launch running the same stages
  *                              separated by grid-wide barriers, sized to the
  *                              batch, with stages that have nothing to do
  *                              skipped (a device without cooperative launch
  *                              uses the chain).
- * Measured on GB300 the two take the same time within a few percent at every
- * batch size (a 1-key call about 35 us, a 64K-key call about 105 us at load
- * factor 0.8): the stages' dependent memory round trips, not the launches,
- * set it.
  * The mode is process-wide; set it while no insert call is being issued.
  * Returns the previous mode, or CKPP_EINVAL for an unknown one. */
 #define CKPP_INSERT_LAUNCH_CHAIN 0

@@ -120,7 +120,7 @@ int ckpp_bulk_insert(ckpp_table* t, const ckpp_key* keys, const uint64_t* vals, 
   if (!n) return CKPP_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
-  if (int rc = prepare_workspace(n, workspace, workspace_bytes, s, ws)) return rc;
+  if (int rc = carve_workspace(n, workspace, workspace_bytes, ws)) return rc;
   return cuda_rc(launch_insert(one_table(t), reinterpret_cast<const uint8_t*>(keys), vals, n, now,
                                (now + ttl) & 0xFFFFu, status, ws, s));
 }
@@ -133,7 +133,7 @@ int ckpp_bulk_delete(ckpp_table* t, const ckpp_key* keys, uint64_t n, uint32_t n
   if (!n) return CKPP_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
-  if (int rc = prepare_workspace(n, workspace, workspace_bytes, s, ws)) return rc;
+  if (int rc = carve_workspace(n, workspace, workspace_bytes, ws)) return rc;
   return cuda_rc(launch_delete(one_table(t), reinterpret_cast<const uint8_t*>(keys), n, now, status, ws, s));
 }
 
@@ -246,7 +246,7 @@ int ckpp_batch_insert(ckpp_batch* b, const ckpp_key* keys, const uint32_t* table
   if (!n) return CKPP_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
-  if (int rc = prepare_workspace(n, workspace, workspace_bytes, s, ws)) return rc;
+  if (int rc = carve_workspace(n, workspace, workspace_bytes, ws)) return rc;
   const TableSet ts{b->host_views[0], b->dev_views, table_ids, (uint32_t)b->tables.size(), b->any_timers ? 1u : 0u};
   return cuda_rc(launch_insert(ts, reinterpret_cast<const uint8_t*>(keys), vals, n, now, (now + ttl) & 0xFFFFu, status,
                                ws, s));
@@ -261,7 +261,7 @@ int ckpp_batch_delete(ckpp_batch* b, const ckpp_key* keys, const uint32_t* table
   if (!n) return CKPP_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
-  if (int rc = prepare_workspace(n, workspace, workspace_bytes, s, ws)) return rc;
+  if (int rc = carve_workspace(n, workspace, workspace_bytes, ws)) return rc;
   const TableSet ts{b->host_views[0], b->dev_views, table_ids, (uint32_t)b->tables.size(), b->any_timers ? 1u : 0u};
   return cuda_rc(launch_delete(ts, reinterpret_cast<const uint8_t*>(keys), n, now, status, ws, s));
 }

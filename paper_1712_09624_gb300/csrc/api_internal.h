@@ -73,7 +73,8 @@ constexpr WsLayout ws_layout(uint64_t n) {
   return L;
 }
 
-inline int prepare_workspace(uint64_t n, void* workspace, size_t bytes, cudaStream_t s, Workspace& ws) {
+// The parts of a caller's workspace; the insert and delete launchers clear what must start at zero.
+inline int carve_workspace(uint64_t n, void* workspace, size_t bytes, Workspace& ws) {
   const WsLayout L = ws_layout(n);
   if (!workspace || bytes < L.total || !aligned(workspace, kAlign)) return CKPP_EINVAL;
   uint8_t* w = static_cast<uint8_t*>(workspace);
@@ -88,7 +89,7 @@ inline int prepare_workspace(uint64_t n, void* workspace, size_t bytes, cudaStre
   ws.m_mask = (uint32_t)(L.m - 1);
   ws.idx_bits = L.idx_bits;
   ws.fix_cap = L.fix_cap;
-  return launch_workspace_clear(ws, s) == cudaSuccess ? CKPP_OK : CKPP_ECUDA;
+  return CKPP_OK;
 }
 
 // Sec. 4.2: a timed call more than 64512 units after the last scan could see

@@ -31,17 +31,19 @@ inline int device_sm_count() {
   return v;
 }
 
-// Words of a workspace's counters. The first 32 bytes are a caller's diagnostics
-// (ckpp_workspace_bytes): list counts of the displacement passes. Counters that
-// one kernel appends to are in lines of their own.
-constexpr uint32_t kCntPending = 0,    // keys phase 1 left (in `pending`)
-    kCntFixup = 1, kCntFixupOverflow = 2,
-                   kCntMoved1 = 3,     // keys the one-move pass left (in `retry`)
-    kCntGrid = 5,                      // keys the grid search left (in `pending`)
-    kCntSecond = 6,                    // keys the second search left (in `retry`)
-    kCntBarrier = 8,                   // two words: the grid barrier of the single-launch insert
-    kCntFollowers = 32, kCntSticky = 64;
-constexpr uint32_t kCounterWords = 128;
+// Words of a workspace's counters. The first 32 bytes are one sector, read at
+// once where several counts are wanted, and a caller's diagnostics
+// (ckpp_workspace_bytes).
+constexpr uint32_t kCntPending = 0;        // keys phase 1 left (in `pending`)
+constexpr uint32_t kCntFixup = 1;          // buckets whose filter may want a reset (in `fixup`)
+constexpr uint32_t kCntFixupOverflow = 2;  // 1: more than `fixup` holds
+constexpr uint32_t kCntMoved1 = 3;         // keys the one-move pass left (in `retry`)
+constexpr uint32_t kCntFollowers = 4;      // repeated keys (in `followers`)
+constexpr uint32_t kCntGrid = 5;           // keys the grid search left (in `pending`)
+constexpr uint32_t kCntSecond = 6;         // keys the second search left (in `retry`)
+constexpr uint32_t kCntSticky = 7;         // claimed bits to clear (in `sticky`)
+constexpr uint32_t kCntBarrier = 8;        // two words: the grid barrier of the single-launch insert
+constexpr uint32_t kCounterWords = 64;
 
 // Device scratch for one insert or delete batch (carved out of the caller's
 // workspace buffer, see ws_layout in api_internal.h). Only the counters and the

@@ -73,10 +73,9 @@ __device__ __forceinline__ uint32_t set_owner(const Workspace& ws, const TableSe
   return i;
 }
 
-// Appending to lists. Every returning atomic on one counter takes 0.8 ns (a
-// warp's append each, of a 1M-key batch: 26 us per list, and twice that for two
-// counters in one 128-byte line), so a block takes its places in all its lists
-// with one atomic per list, and the lists' counters are a line apart.
+// Appending to lists. Every returning atomic on one counter, or on two counters
+// of one 128-byte line, takes 0.8 ns (a warp's append to one list each, of a
+// 1M-key batch: 26 us), so a block takes its places with one atomic per list.
 template <int kLists>
 struct BlockLists {
   uint32_t count[kLists], base[kLists];
@@ -127,9 +126,55 @@ __device__ __forceinline__ void write_follower(const Workspace& ws, uint32_t at,
   ws.range[owner] = make_uint2(owner, owner);
 }
 
+// All counts at once.
+struct Counts {
+  uint32_t c[8];
+  __device__ __forceinline__ uint32_t operator[](uint32_t i) const { return c[i]; }
+};
+
+__device__ __forceinline__ Counts load_counts(const Workspace& ws) {
+  uint64_t w[4];
+  ld256_cg(ws.counters, w);
+  Counts r;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r.c[i] = (uint32_t)(w[i / 2] >> (32 * (i & 1)));
+  return r;
+}
+
+// The workspace of a call that one block runs alone (at most kOneBlockKeys
+// keys), its set, ranges and followers moved to shared memory.
+constexpr uint32_t kOneBlockKeys = 256;
+struct OneBlockSet {
+  __align__(16) uint32_t set[8 * kOneBlockKeys];
+};
+struct OneBlockGroups {
+  uint2 range[kOneBlockKeys], followers[kOneBlockKeys];
+};
+__device__ __forceinline__ Workspace in_shared(Workspace ws, OneBlockSet& set, OneBlockGroups& groups) {
+  ws.set = set.set;
+  ws.range = groups.range;
+  ws.followers = groups.followers;
+  return ws;
+}
+
+// Reset the counters to 0 and the set to empty. (m is a power of two >= 64 and
+// the set 256-byte aligned: whole 16-byte vectors.)
+__device__ __forceinline__ void clear_workspace(const Workspace& ws, uint32_t worker, uint32_t workers) {
+  uint4* set = reinterpret_cast<uint4*>(ws.set);
+  const uint64_t n_vec = ((uint64_t)ws.m_mask + 1) / 4;
+  for (uint32_t j = worker; j < kCounterWords; j += workers) ws.counters[j] = 0u;
+  for (uint64_t j = worker; j < n_vec; j += workers) set[j] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+}
+
+// All threads of the cluster arrive; what each wrote before is seen by all after.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // Widen each follower's group to include it (after the owners' kernel).
-__device__ __forceinline__ void follower_ranges(const Workspace& ws, uint32_t worker, uint32_t workers) {
-  const uint32_t count = ld32_cg(ws.counters + kCntFollowers);
+__device__ __forceinline__ void follower_ranges(const Workspace& ws, uint32_t count, uint32_t worker,
+                                                uint32_t workers) {
   for (uint32_t j = worker; j < count; j += workers) {
     const uint2 f = ws.followers[j];
     atomicMin(&ws.range[f.y].x, f.x);

@@ -117,18 +117,20 @@ __device__ __forceinline__ uint4& row_chunk(P1Rows& R, uint32_t r, uint32_t c) {
 struct P1Bucket {
   uint32_t b, ctrl, match;  // match: busy slots with the key's tag
   uint32_t dead;            // busy slots with a dead entry (timers)
+  uint32_t fresh;           // slots with the expiry that this batch writes (timers; only where match is set)
   uint64_t bloom;
 };
 
 __device__ __forceinline__ P1Bucket p1_bucket(const TableView& t, uint32_t b, const Snap& s, uint32_t tag, bool timers,
-                                              uint32_t now) {
+                                              uint32_t now, uint32_t expiry) {
   P1Bucket r;
   r.b = b;
   r.ctrl = (uint32_t)s.w[3];
   r.match = tag_mask(s.w[0], s.w[1], tag) & r.ctrl & kBusyMask;
   r.bloom = s.w[2];
-  r.dead = 0;
+  r.dead = r.fresh = 0;
   if (timers) {
+    if (r.match) r.fresh = tag_mask(s.e0, s.e1, expiry);
     r.dead = r.ctrl & ~alive_mask(s.e0, s.e1, now) & kBusyMask;
     if (r.dead) {  // read again behind the ctrl word
       fence_acq_rel();
@@ -222,12 +224,14 @@ __device__ __forceinline__ uint8_t p1_stored(const TableView& t, const P1Bucket&
       work = got > 0 ? kP1Revive : kP1None;
       return got > 0 ? kStInserted : got == 0 ? 0 : kStBusy;
     }
-    // The expiry that called the entry alive may be that of a key which has taken
-    // the slot since: then the word shows its claim.
-    fence_acq_rel();
-    if ((ld32_cg(ctrl_ptr(t, r.b)) >> (kClaimShift + sl)) & 1u) {
-      work = kP1None;
-      return 0;
+    // The expiry that called the entry alive may be that of a key of this batch which
+    // has taken the slot since its word was read: then the word shows the claim by now.
+    if ((r.fresh >> sl) & 1u) {
+      fence_acq_rel();
+      if ((ld32_cg(ctrl_ptr(t, r.b)) >> (kClaimShift + sl)) & 1u) {
+        work = kP1None;
+        return 0;
+      }
     }
   }
   return kStUpdated;
@@ -322,7 +326,7 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
   P1Bucket r{}, r2{};
   bool maybe2 = false, have2 = false;
   if (mine) {
-    r = p1_bucket(t, a.b1, s, a.tag, timers, now);
+    r = p1_bucket(t, a.b1, s, a.tag, timers, now, expiry);
     maybe2 = (r.bloom & a.bits) == a.bits;  // the filter allows the secondary
     have2 = maybe2 || !claimable(r.ctrl, r.dead);
   }
@@ -334,7 +338,7 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
   bool sticky = false;
   if (mine) {
     if ((sl = p1_find(t, r, k)) >= 0) st = p1_stored(t, r, (uint32_t)sl, timers, work);
-    if (have2) r2 = p1_bucket(t, a.b2, s, a.tag, timers, now);
+    if (have2) r2 = p1_bucket(t, a.b2, s, a.tag, timers, now, expiry);
     if (!st && maybe2 && (sl = p1_find(t, r2, k)) >= 0) {
       st = p1_stored(t, r2, (uint32_t)sl, timers, work);
       if (st) r = r2;
@@ -367,7 +371,7 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
         // the primary filled up under the claim: its secondary
         if (!have2) {
           p1_fetch_one(t, a.b2, timers, s);
-          r2 = p1_bucket(t, a.b2, s, a.tag, timers, now);
+          r2 = p1_bucket(t, a.b2, s, a.tag, timers, now, expiry);
         }
         r = r2;
       }
@@ -400,17 +404,19 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
   if (sticky) ws.sticky[at[2]] = (unsigned long long)i << 32 | r.b;
 }
 
+constexpr int kP1Threads = 128;
+
 template <bool kTimers>
-__global__ void __launch_bounds__(kThreads, 4) insert_phase1(TableSet ts, const uint8_t* __restrict__ keys,
+__global__ void __launch_bounds__(kP1Threads, 1024 / kP1Threads) insert_phase1(TableSet ts, const uint8_t* __restrict__ keys,
                                                              const uint64_t* __restrict__ vals, uint64_t n,
                                                              uint32_t now, uint32_t expiry,
                                                              uint8_t* __restrict__ status, Workspace ws) {
-  __shared__ P1Rows rows[kThreads / 32];
+  __shared__ P1Rows rows[kP1Threads / 32];
   __shared__ P1Lists lists;
   lists_init(lists);
   pdl_wait();
   pdl_release();
-  const uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x;
+  const uint64_t i = blockIdx.x * (uint64_t)kP1Threads + threadIdx.x;
   phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
 }
 
@@ -905,7 +911,8 @@ __global__ void __launch_bounds__(kThreads) insert_move1(TableSet ts, const uint
                                                          uint32_t* next, uint32_t* next_count) {
   pdl_wait();
   pdl_release();
-  follower_ranges(ws, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  follower_ranges(ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x,
+                  gridDim.x * blockDim.x);
   move1_range(ts, keys, vals, now, expiry, status, ws, list, count_ptr, next, next_count,
               blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
@@ -1070,17 +1077,17 @@ __global__ void __launch_bounds__(kThreadsPerBlock) insert_phase2(TableSet ts, c
 // words; the status bytes and stored values of groups with followers.
 __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict__ keys,
                                    const uint64_t* __restrict__ vals, uint8_t* __restrict__ status,
-                                   const Workspace& ws, uint64_t worker, uint64_t workers) {
+                                   const Workspace& ws, const Counts& counts, uint64_t worker, uint64_t workers) {
   const uint64_t stride = workers;
   const uint64_t i = worker;
-  if (ld32_cg(ws.counters + kCntFixupOverflow)) {  // the list overflowed: scan every bucket of every table
+  if (counts[kCntFixupOverflow]) {  // the list overflowed: scan every bucket of every table
     for (uint32_t tb = 0; tb < ts.n_tables; ++tb) {
       const TableView t = ts.table(tb);
       for (uint64_t b = i; b < t.nb; b += stride)
         if (ld32_cg(moved_ptr(t, (uint32_t)b)) == 0u) st64_cg(bloom_ptr(t, (uint32_t)b), 0ull);
     }
   } else {
-    const uint32_t count = min(ld32_cg(ws.counters + kCntFixup), ws.fix_cap);
+    const uint32_t count = min(counts[kCntFixup], ws.fix_cap);
     for (uint64_t j = i; j < count; j += stride) {
       const unsigned long long e = ws.fixup[j];
       const TableView t = ts.table((uint32_t)(e >> 32));
@@ -1088,17 +1095,19 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
       if (ld32_cg(moved_ptr(t, b)) == 0u) st64_cg(bloom_ptr(t, b), 0ull);
     }
   }
-  const uint32_t sticky = ld32_cg(ws.counters + kCntSticky);
+  const uint32_t sticky = counts[kCntSticky];
   for (uint64_t j = i; j < sticky; j += stride) {
     const unsigned long long e = ws.sticky[j];
     atomicAnd(ctrl_ptr(ts.of(e >> 32), (uint32_t)e), ~(kBusyMask << kClaimShift));
   }
-  const uint32_t followers = ld32_cg(ws.counters + kCntFollowers);
+  const uint32_t followers = counts[kCntFollowers];
+  const bool few = followers <= 16384u;
   for (uint64_t j = i; j < followers; j += stride) {
     const uint2 f = ws.followers[j];
     const uint2 range = ws.range[f.y];
     const bool last = f.x == range.y;  // its value is the one that stays
-    // the buckets of a last occurrence are requested before the owner's outcome is looked at
+    // The buckets of a last occurrence are requested before the owner's outcome is looked at, both
+    // at once where there are so few that the time of one counts and not their requests.
     TableView t{};
     Key k{0, 0};
     Addr a{};
@@ -1108,7 +1117,7 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
       k = load_key(keys, f.x);
       a = address_of(k, t.nb, t.seed);
       ld256_cg(bucket_ptr(t, a.b1), s1.w);
-      ld256_cg(bucket_ptr(t, a.b2), s2.w);
+      if (few) ld256_cg(bucket_ptr(t, a.b2), s2.w);
     }
     // the owner's outcome; the group's lowest index takes it over (from INSERTED the owner then
     // becomes UPDATED, which every other follower reports for either)
@@ -1122,6 +1131,7 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
     status[f.x] = st;
     if (last && stored) {
       const int in1 = find_key(t, a.b1, (uint32_t)s1.w[3], s1, k, a.tag);
+      if (in1 < 0 && !few) ld256_cg(bucket_ptr(t, a.b2), s2.w);
       const int in2 = in1 >= 0 ? -1 : find_key(t, a.b2, (uint32_t)s2.w[3], s2, k, a.tag);
       if (in1 >= 0) st64_cg(value_ptr(t, a.b1, in1), vals[f.x]);
       if (in2 >= 0) st64_cg(value_ptr(t, a.b2, in2), vals[f.x]);
@@ -1134,20 +1144,24 @@ __global__ void __launch_bounds__(kThreads) insert_fixup_finish(TableSet ts, con
                                                                 uint8_t* __restrict__ status, Workspace ws) {
   pdl_wait();
   pdl_release();
-  fixup_finish_range(ts, keys, vals, status, ws, blockIdx.x * (uint64_t)blockDim.x + threadIdx.x,
+  fixup_finish_range(ts, keys, vals, status, ws, load_counts(ws), blockIdx.x * (uint64_t)blockDim.x + threadIdx.x,
                      (uint64_t)gridDim.x * blockDim.x);
 }
 
 // --------------------------------------------------- single-launch insert
-// The whole insert call of a small batch in one cooperative launch: the
-// stages of the chain above (phase 1, the one-move pass, the three search
-// passes, fixup and finish) run in order, separated by a
-// grid barrier instead of kernel boundaries. A small batch spends most of a
-// chain's time in the chain's seven dependent launches (each one's start and
-// drain); here it pays two (the workspace clear and this kernel). All blocks
-// are resident at once (cooperative launch, grid sized by the occupancy the
-// kernel reaches), so the barrier cannot wait on a block that has not
-// started. Search queues live in 48 KB of dynamic shared memory per block: the
+// The whole insert call in one launch, the stages of the chain above in order
+// with a barrier between them instead of a kernel boundary. A stage whose list
+// is empty is skipped with its barrier. Two forms:
+//   a cluster     (the default for small batches) one cluster of up to eight
+//                 blocks, which clears the workspace as well: a small batch
+//                 spends most of a chain's time in the starts and drains of the
+//                 chain's eight dependent launches, each also 1.9 us of host
+//                 time, and a cluster's barrier takes a fraction of either;
+//   a whole grid  (CKPP_INSERT_LAUNCH_SINGLE, any size) a cooperative launch
+//                 on a grid sized to the batch, after the workspace clear. All
+//                 blocks are resident at once, so the barrier cannot wait on a
+//                 block that has not started.
+// Search queues live in 48 KB of dynamic shared memory per block: the
 // grid pass runs on 64 threads of every block (96 nodes each; on every warp
 // for a short list), the second pass
 // on every warp (192 nodes and a visited set each), the last on the first warp
@@ -1159,7 +1173,7 @@ constexpr unsigned kSingleMinBlocks = 8;
 // the bounded lock waits a stage may contain, so a barrier gives up only if a block never arrives.
 constexpr int kBarrierSpins = 1 << 22;
 
-static_assert((kSingleThreads / 32) * sizeof(P1Rows) <= kSingleSmem, "phase 1 rows exceed the shared memory");
+static_assert((kSingleThreads / 32) * sizeof(P1Rows) + sizeof(P1Lists) <= kSingleSmem, "phase 1 rows exceed the shared memory");
 static_assert(96 * 64 * sizeof(Node) <= kSingleSmem, "grid pass queues exceed the shared memory");
 static_assert((kSingleThreads / 32) * warp_search_bytes<96>() <= kSingleSmem,
               "grid pass state (one warp per key) exceeds the shared memory");
@@ -1204,80 +1218,109 @@ __device__ bool grid_barrier(uint32_t* count, uint32_t* gen) {
   return ok_s != 0;
 }
 
+// The barrier between two stages of either form.
+template <bool kCluster>
+__device__ __forceinline__ bool stage_barrier(const Workspace& ws) {
+  if constexpr (kCluster) {
+    cluster_barrier();
+    return true;
+  } else {
+    return grid_barrier(ws.counters + kCntBarrier, ws.counters + kCntBarrier + 1);
+  }
+}
+
+// A cluster of one block keeps the set and the groups of equal keys in shared
+// memory: the set before the queues need the room, the groups behind them.
+constexpr size_t kOneSetAt = 20 * 1024, kOneGroupsAt = kSingleSmem - sizeof(OneBlockGroups);
+static_assert((kSingleThreads / 32) * sizeof(P1Rows) + sizeof(P1Lists) <= kOneSetAt &&
+                  kOneSetAt + sizeof(OneBlockSet) <= kOneGroupsAt &&
+                  (kSingleThreads / 32) * warp_search_bytes<192>() <= kOneGroupsAt &&
+                  (kSingleThreads / 32) * warp_search_bytes<96>() <= kOneGroupsAt &&
+                  warp_search_bytes<2048>() <= kOneGroupsAt && kOneBlockKeys <= kGridWarpKeys,
+              "one block's set and groups do not fit beside the queues");
+static_assert(kOneBlockKeys == kSingleThreads, "cluster_blocks gives batches that fit one block a cluster of one");
+
+template <bool kCluster, bool kTimers>
 __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableSet ts, const uint8_t* __restrict__ keys,
                                                                          const uint64_t* __restrict__ vals, uint64_t n,
                                                                          uint32_t now, uint32_t expiry,
-                                                                         uint8_t* __restrict__ status, Workspace ws) {
+                                                                         uint8_t* __restrict__ status,
+                                                                         Workspace caller_ws) {
   extern __shared__ __align__(128) uint8_t smem[];
-  uint32_t* bar_count = ws.counters + kCntBarrier;
-  uint32_t* bar_gen = ws.counters + kCntBarrier + 1;
-  const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
+  const uint32_t tid = blockIdx.x * kSingleThreads + threadIdx.x;
+  const uint32_t threads = gridDim.x * kSingleThreads;
+  const Workspace ws = kCluster && gridDim.x == 1
+                           ? in_shared(caller_ws, *reinterpret_cast<OneBlockSet*>(smem + kOneSetAt),
+                                       *reinterpret_cast<OneBlockGroups*>(smem + kOneGroupsAt))
+                           : caller_ws;
   bool ok = true;
-  P1Rows* rows = reinterpret_cast<P1Rows*>(smem);
-  __shared__ P1Lists lists;
+  if (kCluster) {
+    clear_workspace(ws, tid, threads);
+    stage_barrier<kCluster>(ws);
+  }
+  P1Rows* rows = reinterpret_cast<P1Rows*>(smem);  // phase 1's part of the shared memory, before the queues'
+  P1Lists& lists = *reinterpret_cast<P1Lists*>(rows + kSingleThreads / 32);
   lists_init(lists);
   for (uint64_t first = blockIdx.x * (uint64_t)kSingleThreads; first < n; first += threads) {  // whole blocks
     const uint64_t i = first + threadIdx.x;
-    phase1_one<true>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
+    phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
   }
-  ok &= grid_barrier(bar_count, bar_gen);
-  if (ld32_cg(ws.counters + kCntFollowers)) {
-    follower_ranges(ws, (uint32_t)tid, (uint32_t)threads);
-    if (!ld32_cg(ws.counters + kCntPending)) ok &= grid_barrier(bar_count, bar_gen);
+  ok &= stage_barrier<kCluster>(ws);
+  // lists as in the chain: pending -> one move -> retry -> grid search -> pending -> second pass ->
+  // retry -> last pass. A pass whose list is empty is skipped with its barrier, and so are the ones
+  // after it; every block reads the same counts (final before the barrier), so all skip alike.
+  Counts counts = load_counts(ws);
+  if (counts[kCntFollowers]) {
+    follower_ranges(ws, counts[kCntFollowers], tid, threads);
+    if (!counts[kCntPending]) ok &= stage_barrier<kCluster>(ws);
   }
-  // lists as in the chain: pending [0] -> one move -> retry [3] -> grid search -> pending [5] ->
-  // second pass -> retry [6] -> last pass. A pass whose list is empty is skipped with its barrier;
-  // every block reads the same count (final before the barrier), so all skip alike.
-  if (ld32_cg(ws.counters + kCntPending)) {
-    move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, ws.counters + kCntPending, ws.retry, ws.counters + kCntMoved1,
-                (uint32_t)tid, (uint32_t)threads);
-    ok &= grid_barrier(bar_count, bar_gen);
-  }
-  Node* nodes = reinterpret_cast<Node*>(smem);
-  const uint32_t w = threadIdx.x >> 5;
-  if (const uint32_t listed = ld32_cg(ws.counters + kCntMoved1)) {
-    if (listed <= kGridWarpKeys) {  // a short list: one warp per key
-      uint8_t* mine = smem + w * warp_search_bytes<96>();
-      phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                               ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
-                               reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)),
-                               blockIdx.x * (kSingleThreads / 32) + w, gridDim.x * (kSingleThreads / 32));
-    } else if (threadIdx.x < 64) {
-      const Queue q{nodes + threadIdx.x, 64};
-      phase2_range<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                          ws.counters + kCntGrid, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
+  if (counts[kCntPending]) {
+    Node* nodes = reinterpret_cast<Node*>(smem);
+    const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kSingleThreads / 32) + w;
+    const uint32_t warps = gridDim.x * (kSingleThreads / 32);
+    move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, ws.counters + kCntPending, ws.retry,
+                ws.counters + kCntMoved1, tid, threads);
+    ok &= stage_barrier<kCluster>(ws);
+    counts = load_counts(ws);
+    if (const uint32_t listed = counts[kCntMoved1]) {
+      if (listed <= kGridWarpKeys) {  // a short list: one warp per key
+        uint8_t* mine = smem + w * warp_search_bytes<96>();
+        phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
+                                 ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
+                                 reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)), warp, warps);
+      } else if (threadIdx.x < 64) {
+        const Queue q{nodes + threadIdx.x, 64};
+        phase2_range<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
+                            ws.counters + kCntGrid, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
+      }
+      ok &= stage_barrier<kCluster>(ws);
+      counts = load_counts(ws);
     }
-    ok &= grid_barrier(bar_count, bar_gen);
+    if (const uint32_t listed = counts[kCntGrid]) {
+      uint8_t* mine = smem + w * warp_search_bytes<192>();
+      phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, listed, ws.retry,
+                                ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
+                                reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)), warp, warps);
+      ok &= stage_barrier<kCluster>(ws);
+      counts = load_counts(ws);
+    }
+    if (const uint32_t listed = counts[kCntSecond]) {
+      if (w == 0)
+        phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, (uint32_t*)nullptr,
+                                   (uint32_t*)nullptr, kLastPassKeys, nodes,
+                                   reinterpret_cast<uint32_t*>(smem + 2048 * sizeof(Node)), blockIdx.x, gridDim.x);
+      ok &= stage_barrier<kCluster>(ws);
+      counts = load_counts(ws);
+    }
   }
-  if (ld32_cg(ws.counters + kCntGrid)) {
-    constexpr size_t kPer = warp_search_bytes<192>();
-    uint8_t* mine = smem + w * kPer;
-    phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, ld32_cg(ws.counters + kCntGrid), ws.retry,
-                              ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
-                              reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)),
-                              blockIdx.x * (kSingleThreads / 32) + w, gridDim.x * (kSingleThreads / 32));
-    ok &= grid_barrier(bar_count, bar_gen);
-  }
-  if (ld32_cg(ws.counters + kCntSecond)) {
-    if (w == 0)
-      phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, ld32_cg(ws.counters + kCntSecond),
-                                 (uint32_t*)nullptr, (uint32_t*)nullptr, kLastPassKeys, nodes,
-                                 reinterpret_cast<uint32_t*>(smem + 2048 * sizeof(Node)), blockIdx.x, gridDim.x);
-    ok &= grid_barrier(bar_count, bar_gen);
-  }
-  fixup_finish_range(ts, keys, vals, status, ws, tid, threads);
+  fixup_finish_range(ts, keys, vals, status, ws, counts, tid, threads);
   if (!ok && threadIdx.x == 0) latch_error(ts.table(0), kErrLockTimeout);
 }
 
 // ------------------------------------------------------- workspace reset
-__global__ void __launch_bounds__(kThreads) workspace_clear(uint32_t* __restrict__ counters,
-                                                            uint4* __restrict__ set, uint64_t n_vec) {
+__global__ void __launch_bounds__(kThreads) workspace_clear(Workspace ws) {
   pdl_release();
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (tid < kCounterWords) counters[tid] = 0u;
-  for (uint64_t j = tid; j < n_vec; j += stride) set[j] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+  clear_workspace(ws, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads);
 }
 
 }  // namespace
@@ -1288,8 +1331,7 @@ cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s) {
   const uint64_t want = n_vec > kCounterWords ? n_vec : kCounterWords;
   const uint64_t blocks = (want + kThreads - 1) / kThreads;
   const uint64_t cap = 16ull * device_sm_count();
-  workspace_clear<<<(unsigned)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(
-      ws.counters, reinterpret_cast<uint4*>(ws.set), n_vec);
+  workspace_clear<<<(unsigned)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(ws);
   return cudaGetLastError();
 }
 
@@ -1311,7 +1353,8 @@ int single_launch_blocks_per_sm() {
   if (v) return v > 0 ? v : 0;
   int coop = 0, per_sm = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, insert_single_launch, kSingleThreads, kSingleSmem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, insert_single_launch<false, true>, kSingleThreads,
+                                                    kSingleSmem) !=
           cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -1338,7 +1381,7 @@ cudaError_t launch_single(const TableSet& ts, const uint8_t* keys, const uint64_
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, insert_single_launch, ts, keys, vals, n, now, expiry, status, ws);
+  return cudaLaunchKernelEx(&cfg, insert_single_launch<false, true>, ts, keys, vals, n, now, expiry, status, ws);
 }
 
 }  // namespace
@@ -1351,13 +1394,22 @@ int set_insert_launch(int mode) {
 cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_t* vals, uint64_t n, uint32_t now,
                           uint32_t expiry, uint8_t* status, const Workspace& ws, cudaStream_t s) {
   const int mode = g_insert_launch.load(std::memory_order_relaxed);
+  cudaError_t e;
   if (mode == kInsertLaunchSingle) {
     const int per_sm = single_launch_blocks_per_sm();
-    if (per_sm > 0) return launch_single(ts, keys, vals, n, now, expiry, status, ws, s, per_sm);
+    if (per_sm > 0) {
+      e = launch_workspace_clear(ws, s);
+      return e != cudaSuccess ? e : launch_single(ts, keys, vals, n, now, expiry, status, ws, s, per_sm);
+    }
+  } else if (n <= kClusterKeys) {
+    return launch_cluster(ts.any_timers ? insert_single_launch<true, true> : insert_single_launch<true, false>, false,
+                          cluster_blocks(n, kSingleThreads), kSingleThreads, kSingleSmem, s, ts, keys, vals, n, now,
+                          expiry, status, ws);
   }
+  e = launch_workspace_clear(ws, s);
+  if (e != cudaSuccess) return e;
   const unsigned sms = (unsigned)device_sm_count();
-  cudaError_t e;
-  e = launch_chained(ts.any_timers ? insert_phase1<true> : insert_phase1<false>, grid_for(n, kThreads), kThreads, s, ts,
+  e = launch_chained(ts.any_timers ? insert_phase1<true> : insert_phase1<false>, grid_for(n, kP1Threads), kP1Threads, s, ts,
                      keys, vals, n, now, expiry, status, ws);
   if (e != cudaSuccess) return e;
   // lists: phase 1 -> pending [0] -> move1 -> retry [3] -> grid search ->

@@ -65,9 +65,9 @@ extern "C" int ckpp_bulk_insert_noalloc(ckpp_table* t, const ckpp_key* keys, con
   if (int rc = scratch_address(&scratch)) return rc;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Workspace ws;
-  // prepare_workspace clears the counters and the duplicate-key set, the parts
+  // launch_insert clears the counters and the duplicate-key set, the parts
   // that must start at zero (the array keeps the previous call's contents).
-  if (int rc = prepare_workspace(n, scratch, kNoallocBytes, s, ws)) return rc;
+  if (int rc = carve_workspace(n, scratch, kNoallocBytes, ws)) return rc;
   return cuda_rc(launch_insert(one_table(t), reinterpret_cast<const uint8_t*>(keys), vals, n, now,
                                (now + ttl) & 0xFFFFu, status, ws, s));
 }
