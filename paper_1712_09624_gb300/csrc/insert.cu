@@ -831,7 +831,7 @@ __device__ int execute_move1(const TableView& t, uint32_t tid, uint32_t x, uint3
   return ok ? 1 : 0;
 }
 
-// One-move pass over `list` (count in *count_ptr): for each key, the entries
+// One-move pass over list[0..count): for each key, the entries
 // of b1 and then of b2 are read with the buckets they can move to (two memory
 // round trips per root: the root's keys and control word, then the control
 // words of the buckets its entries can move to; each entry's other bucket
@@ -842,9 +842,8 @@ __device__ int execute_move1(const TableView& t, uint32_t tid, uint32_t x, uint3
 // worker / workers: this thread's index among the threads sharing the pass.
 __device__ void move1_range(const TableSet& ts, const uint8_t* __restrict__ keys, const uint64_t* __restrict__ vals,
                             uint32_t now, uint32_t expiry, uint8_t* __restrict__ status, const Workspace& ws,
-                            const uint32_t* list, const uint32_t* count_ptr, uint32_t* next, uint32_t* next_count,
+                            const uint32_t* list, uint32_t count, uint32_t* next, uint32_t* next_count,
                             uint32_t worker, uint32_t workers) {
-  const uint32_t count = ld32_cg(count_ptr);
   for (uint32_t j = worker; j < count; j += workers) {
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
@@ -904,7 +903,66 @@ __device__ void move1_range(const TableSet& ts, const uint8_t* __restrict__ keys
   }
 }
 
-__global__ void __launch_bounds__(kThreads) insert_move1(TableSet ts, const uint8_t* __restrict__ keys,
+// The same pass with half a warp per key, for a list so short that the time of
+// one key sets the pass's: lane r * 8 + sl of the half reads slot sl of root r,
+// so that both roots' keys come in one round trip and all 16 buckets their
+// entries can move to in a second, where a thread takes up to ten. The first
+// one with room, in the thread form's order, is the path; its lane executes it.
+// half / halves: this half warp's index among those sharing the pass (whole
+// warps call this).
+__device__ void move1_range_half(const TableSet& ts, const uint8_t* __restrict__ keys,
+                                 const uint64_t* __restrict__ vals, uint32_t now, uint32_t expiry,
+                                 uint8_t* __restrict__ status, const Workspace& ws, const uint32_t* list,
+                                 uint32_t count, uint32_t* next, uint32_t* next_count, uint32_t half,
+                                 uint32_t halves) {
+  const uint32_t lane = threadIdx.x & 15u, sl = lane & 7u;
+  const uint32_t shift = threadIdx.x & 16u;  // of this half's lanes in a ballot
+  for (uint32_t first = half & ~1u; first < count; first += halves) {  // the same for both halves
+    const uint32_t j = first + (half & 1u);
+    const bool act = j < count;
+    const uint32_t i = act ? list[j] : 0u;
+    TableView t{};
+    Key k{0, 0};
+    uint64_t v = 0;
+    Addr a{};
+    uint32_t x = 0, y = 0, f = 0;
+    if (act) {
+      t = ts.of(i);
+      v = vals[i];
+      k = load_key(keys, i);
+      a = address_of(k, t.nb, t.seed);
+      x = lane < 8u ? a.b1 : a.b2;
+      const uint32_t cr = ld32_cg(ctrl_ptr(t, x));
+      Key e;
+      ld128_cg(key_ptr(t, x, sl), e.k0, e.k1);
+      y = other_bucket(e, x, (cr >> (kInsecShift + sl)) & 1u, t.nb, t.seed);
+      Snap s;
+      const uint32_t cy = ld32_cg(ctrl_ptr(t, y));
+      s.e0 = s.e1 = 0;
+      if (t.timers) ld128_cg(expiry_ptr(t, y, 0), s.e0, s.e1);
+      if (y != a.b1 && y != a.b2) f = free_mask(t, cy, s, now);  // the roots have no room
+    }
+    const uint32_t with_room = (__ballot_sync(kWarpAll, f != 0u) >> shift) & 0xFFFFu;
+    if (act && (with_room ? lane == (uint32_t)__ffs(with_room) - 1u : lane == 0u)) {
+      int rc = 0;
+      if (with_room) rc = execute_move1(t, ts.id(i), x, sl, y, __ffs(f) - 1, k, v, a, now, expiry, ws);
+      if (rc == 0) {
+        next[atomicAdd(next_count, 1u)] = i;
+      } else {
+        if (rc < 0) latch_error(t, kErrLockTimeout);
+        status[i] = rc > 0 ? kStInserted : kStBusy;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// The longest list that runs half a warp per key (if there are as many halves):
+// a list of 4.9K keys of a 134M-slot table 28 -> 19 us, of 7K keys with timers 22
+// -> 20 us; 13K keys 82 -> 84 us of a whole call, 55K keys 115 -> 147 us.
+constexpr uint32_t kMoveHalfKeys = 8192;
+
+__global__ void __launch_bounds__(kThreads, 1) insert_move1(TableSet ts, const uint8_t* __restrict__ keys,
                                                          const uint64_t* __restrict__ vals, uint32_t now,
                                                          uint32_t expiry, uint8_t* __restrict__ status, Workspace ws,
                                                          const uint32_t* list, const uint32_t* count_ptr,
@@ -913,8 +971,14 @@ __global__ void __launch_bounds__(kThreads) insert_move1(TableSet ts, const uint
   pdl_release();
   follower_ranges(ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x,
                   gridDim.x * blockDim.x);
-  move1_range(ts, keys, vals, now, expiry, status, ws, list, count_ptr, next, next_count,
-              blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  const uint32_t worker = blockIdx.x * blockDim.x + threadIdx.x, workers = gridDim.x * blockDim.x;
+  const uint32_t count = ld32_cg(count_ptr);
+  if (count <= min(kMoveHalfKeys, workers / 16u)) {
+    move1_range_half(ts, keys, vals, now, expiry, status, ws, list, count, next, next_count, worker / 16u,
+                     workers / 16u);
+  } else {
+    move1_range(ts, keys, vals, now, expiry, status, ws, list, count, next, next_count, worker, workers);
+  }
 }
 
 // Displacement pass over `list` (count in *count). Keys that find no path
@@ -1278,8 +1342,13 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
     Node* nodes = reinterpret_cast<Node*>(smem);
     const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kSingleThreads / 32) + w;
     const uint32_t warps = gridDim.x * (kSingleThreads / 32);
-    move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, ws.counters + kCntPending, ws.retry,
-                ws.counters + kCntMoved1, tid, threads);
+    if (counts[kCntPending] <= min(kMoveHalfKeys, threads / 16u)) {
+      move1_range_half(ts, keys, vals, now, expiry, status, ws, ws.pending, counts[kCntPending], ws.retry,
+                       ws.counters + kCntMoved1, tid / 16u, threads / 16u);
+    } else {
+      move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, counts[kCntPending], ws.retry,
+                  ws.counters + kCntMoved1, tid, threads);
+    }
     ok &= stage_barrier<kCluster>(ws);
     counts = load_counts(ws);
     if (const uint32_t listed = counts[kCntMoved1]) {
@@ -1419,7 +1488,7 @@ cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_
     const uint64_t want = (n + keys_per_block - 1) / keys_per_block;
     return want < blocks ? (unsigned)want : blocks;
   };
-  e = launch_chained(insert_move1, cap(sms * 16, kThreads), kThreads, s, ts, keys, vals, now, expiry, status, ws,
+  e = launch_chained(insert_move1, cap(sms * 16, kThreads / 16), kThreads, s, ts, keys, vals, now, expiry, status, ws,
                      (const uint32_t*)ws.pending, (const uint32_t*)(ws.counters + kCntPending), ws.retry, ws.counters + kCntMoved1);
   if (e != cudaSuccess) return e;
   e = launch_chained(insert_phase2<kP2Threads, 96, 4>, cap(sms * 4, kP2Threads / 32), kP2Threads, s, ts, keys, vals, now, expiry, status,
