@@ -187,7 +187,7 @@ struct ckpp_batch {
   std::vector<ckpp_table*> tables;
   std::vector<TableView> host_views;  // kept alive for the copy to the device
   TableView* dev_views;
-  unsigned long long* ctrl;           // the lookup kernel's chunk and finished-warp counters
+  unsigned long long* ctrl;           // the lookup kernel's chunk and finished-block counters
   bool any_timers;                    // some table has timers
   int sms;
 };

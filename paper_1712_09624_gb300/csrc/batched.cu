@@ -14,7 +14,7 @@
 // job of its previous key (keys are drawn in increasing order), and the warp
 // runs the cooperative lookup of probe.cuh over keys of possibly different
 // tables.
-// The last warp to finish resets the counter for the next launch, so
+// The last block to finish resets the counter for the next launch, so
 // launches that use one batch descriptor must not overlap on the GPU.
 // Tuning (picked by the autotuner):
 //   threads per key  1, 2 or 4 lanes of the warp per key in an iteration:
@@ -43,15 +43,25 @@ struct BatchJob {  // layout of ckpp_lookup_job
 namespace {
 
 constexpr int kBatchThreads = 512;  // 16 warps share one copy of the job prefix array
-constexpr unsigned long long kMaxChunksPerDraw = 8;
+constexpr uint32_t kMaxChunksPerDraw = 8;
 
-// Exclusive prefix sums of the first nj job sizes into prefix[0..nj].
-__device__ void scan_jobs(const BatchJob* __restrict__ jobs, uint32_t nj, unsigned long long* prefix) {
+// The number of jobs nj (*n_jobs, clamped to max_jobs), and the exclusive prefix
+// sums of their sizes in prefix[0..nj].
+__device__ uint32_t scan_jobs(const BatchJob* __restrict__ jobs, const uint32_t* __restrict__ n_jobs,
+                              uint32_t max_jobs, unsigned long long* prefix) {
   __shared__ unsigned long long warp_sums[kBatchThreads / 32];
+  // with a job per thread at most, the sizes are requested together with the count
+  const bool one_each = max_jobs <= blockDim.x;
+  const uint32_t mine = one_each && threadIdx.x < max_jobs ? jobs[threadIdx.x].n : 0u;
+  const uint32_t nj = n_jobs ? min(ld32_cg(n_jobs), max_jobs) : max_jobs;
   const uint32_t per = (nj + blockDim.x - 1) / blockDim.x;
   const uint32_t lo = min(nj, threadIdx.x * per), hi = min(nj, lo + per);
   unsigned long long local = 0;
-  for (uint32_t j = lo; j < hi; ++j) local += jobs[j].n;
+  if (one_each) {
+    local = threadIdx.x < nj ? mine : 0u;
+  } else {
+    for (uint32_t j = lo; j < hi; ++j) local += jobs[j].n;
+  }
   // inclusive warp scan of the per-thread sums
   unsigned long long x = local;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -73,12 +83,18 @@ __device__ void scan_jobs(const BatchJob* __restrict__ jobs, uint32_t nj, unsign
   }
   __syncthreads();
   unsigned long long run = x - local + (warp ? warp_sums[warp - 1] : 0);
-  for (uint32_t j = lo; j < hi; ++j) {
-    prefix[j] = run;
-    run += jobs[j].n;
+  if (one_each) {
+    if (threadIdx.x < nj) prefix[threadIdx.x] = run;
+    run += local;
+  } else {
+    for (uint32_t j = lo; j < hi; ++j) {
+      prefix[j] = run;
+      run += jobs[j].n;
+    }
   }
   if (threadIdx.x == blockDim.x - 1) prefix[nj] = run;
   __syncthreads();
+  return nj;
 }
 
 // Index of the job holding flat key idx: the last j with prefix[j] <= idx,
@@ -171,37 +187,47 @@ __global__ void __launch_bounds__(kBatchThreads) batched_lookup_kernel(const Tab
   extern __shared__ __align__(128) unsigned long long prefix[];
   WarpStage<G>* stages =
       reinterpret_cast<WarpStage<G>*>(reinterpret_cast<uint8_t*>(prefix) + stage_offset(max_jobs));
-  const uint32_t nj = n_jobs_ptr ? min(ld32_cg(n_jobs_ptr), max_jobs) : max_jobs;
-  scan_jobs(jobs, nj, prefix);
+  const uint32_t nj = scan_jobs(jobs, n_jobs_ptr, max_jobs, prefix);
   const unsigned long long total = prefix[nj];
   const uint64_t pol = policy_evict_first();
   const uint32_t lane = threadIdx.x & 31;
-  const unsigned long long per_chunk = (unsigned long long)kpw * G;
-  const unsigned long long chunks = (total + per_chunk - 1) / per_chunk;
-  // Chunks per atomic draw: up to kMaxChunksPerDraw on large launches (one
-  // counter word serves every warp of the grid), fewer on small ones, so that
-  // every warp gets about four draws rather than a few warps all the work.
-  const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-  unsigned long long per_draw = chunks / (4 * warps);
-  per_draw = per_draw < 1 ? 1 : (per_draw > kMaxChunksPerDraw ? kMaxChunksPerDraw : per_draw);
+  const uint32_t per_chunk = kpw * G;
+  // Chunks per draw: up to kMaxChunksPerDraw on large launches (one counter
+  // word serves every warp of the grid), fewer on small ones, so that every
+  // warp gets about four draws rather than a few warps all the work.
+  const uint32_t warps = gridDim.x * (kBatchThreads >> 5);
+  const unsigned long long quarter = total / per_chunk / (4ull * warps);
+  const uint32_t per_draw =
+      per_chunk * (quarter < 1 ? 1u : quarter > kMaxChunksPerDraw ? kMaxChunksPerDraw : (uint32_t)quarter);  // keys
+  // Every warp's first draw is its own index; only a launch with more draws than
+  // warps has its warps draw the rest from the counter. (The 4864 warps of two
+  // blocks per SM each drawing twice and counting themselves out, 0.8 ns per
+  // atomic on one line, were most of a small launch's time: 48 jobs of 40K keys
+  // in all 13.3 us, now 8.2.)
+  const bool more = total > (unsigned long long)warps * per_draw;
   uint32_t hint = 0;  // chunks are drawn in increasing order, so a lane's keys only move forward
-  for (;;) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(ctrl, 1ull) * per_draw;
-    c = __shfl_sync(kFull, c, 0);
-    if (c >= chunks) break;
-    const unsigned long long c_end = c + per_draw < chunks ? c + per_draw : chunks;
-    for (; c < c_end; ++c)
-      lookup_chunk<G, kTM>(tables, n_tables, jobs, prefix, nj, total, c * per_chunk, kpw, now, pol, hint,
+  unsigned long long at = (unsigned long long)(blockIdx.x * (kBatchThreads >> 5) + (threadIdx.x >> 5)) * per_draw;
+  while (at < total) {
+#pragma unroll 1
+    for (uint32_t k = 0; k < per_draw && at + k < total; k += per_chunk)
+      lookup_chunk<G, kTM>(tables, n_tables, jobs, prefix, nj, total, at + k, kpw, now, pol, hint,
                            stages[threadIdx.x >> 5]);
+    if (!more) break;
+    unsigned long long drawn = 0;
+    if (lane == 0) drawn = atomicAdd(ctrl, 1ull);
+    at = (warps + __shfl_sync(kFull, drawn, 0)) * per_draw;
   }
-  // Every warp has drawn past the last chunk before it counts itself out, so
-  // the last one out can reset the counters for the next launch.
-  if (lane == 0) {
-    unsigned int* out = reinterpret_cast<unsigned int*>(ctrl + 1);
-    if (atomicAdd(out, 1u) == (unsigned int)(warps - 1)) {
-      atomicExch(ctrl, 0ull);
-      atomicExch(out, 0u);
+  // Every warp of a block has drawn past the last chunk before the block
+  // counts itself out, so the last one out can reset the counters for the next
+  // launch.
+  if (more) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned int* out = reinterpret_cast<unsigned int*>(ctrl + 1);
+      if (atomicAdd(out, 1u) == gridDim.x - 1) {
+        atomicExch(ctrl, 0ull);
+        atomicExch(out, 0u);
+      }
     }
   }
 }

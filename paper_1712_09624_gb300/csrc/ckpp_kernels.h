@@ -94,7 +94,7 @@ cudaError_t launch_probe_counts(const TableView& t, const uint8_t* keys, uint64_
 
 // Batched form (batched.cu): tables [n_tables] in device memory, jobs a device
 // array of ckpp_lookup_job, n_jobs NULL or a device count (clamped to max_jobs),
-// ctrl the descriptor's two zeroed counter words (chunk counter, warps done).
+// ctrl the descriptor's two zeroed counter words (chunk counter, blocks done).
 cudaError_t prepare_batched_lookup();
 cudaError_t launch_batched_lookup(const TableView* tables, uint32_t n_tables, const void* jobs, const uint32_t* n_jobs,
                                   uint32_t max_jobs, uint32_t now, int threads_per_key, int group_depth,
