@@ -1582,7 +1582,8 @@ cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_
     const uint64_t want = (n + keys_per_block - 1) / keys_per_block;
     return want < blocks ? (unsigned)want : blocks;
   };
-  e = launch_chained(insert_move1, cap(sms * 16, kThreads / 16), kThreads, s, ts, keys, vals, now, expiry, status, ws,
+  const unsigned by_thread = cap(sms * 16, kThreads), by_half = cap(kMoveHalfKeys / (kThreads / 16), kThreads / 16);
+  e = launch_chained(insert_move1, by_thread > by_half ? by_thread : by_half, kThreads, s, ts, keys, vals, now, expiry, status, ws,
                      (const uint32_t*)ws.pending, (const uint32_t*)(ws.counters + kCntPending), ws.retry, ws.counters + kCntMoved1);
   if (e != cudaSuccess) return e;
   e = launch_chained(insert_phase2<kP2Threads, 96, 4>, cap(sms * 4, kP2Threads / 32), kP2Threads, s, ts, keys, vals, now, expiry, status,
