@@ -86,6 +86,7 @@ inline int carve_workspace(uint64_t n, void* workspace, size_t bytes, Workspace&
   ws.retry = reinterpret_cast<uint32_t*>(w + L.off_retry);
   ws.sticky = reinterpret_cast<unsigned long long*>(w + L.off_sticky);
   ws.fixup = reinterpret_cast<unsigned long long*>(w + L.off_fixup);
+  ws.n = (uint32_t)n;
   ws.m_mask = (uint32_t)(L.m - 1);
   ws.idx_bits = L.idx_bits;
   ws.fix_cap = L.fix_cap;

@@ -42,11 +42,10 @@ inline unsigned cluster_blocks(uint64_t n, int threads) {
   return blocks;
 }
 
-// chained: as launch_chained.
 template <typename... Params, typename... Args>
-cudaError_t launch_cluster(void (*kernel)(Params...), bool chained, unsigned blocks, unsigned block, size_t smem,
+cudaError_t launch_cluster(void (*kernel)(Params...), unsigned blocks, unsigned block, size_t smem,
                            cudaStream_t s, Args... args) {
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = blocks;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
@@ -55,10 +54,8 @@ cudaError_t launch_cluster(void (*kernel)(Params...), bool chained, unsigned blo
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = chained ? 2 : 1;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

@@ -46,19 +46,22 @@ constexpr uint32_t kCntBarrier = 8;        // two words: the grid barrier of the
 constexpr uint32_t kCounterWords = 64;
 
 // Device scratch for one insert or delete batch (carved out of the caller's
-// workspace buffer, see ws_layout in api_internal.h). Only the counters and the
-// set are cleared before a call; every other word is written before it is read.
+// workspace buffer, see ws_layout in api_internal.h). The counters, the set and
+// the ranges are cleared before a call; every other word is written before it is
+// read.
 struct Workspace {
   uint32_t* counters;   // list counts (kCnt*)
   uint32_t* set;        // [m] open-addressing set of batch keys (dedup.cuh): hash bits << idx_bits | batch index of
                         // the key that claimed the position, or kEmpty
-  uint2* range;         // [n] lowest and highest batch index of the group of key i, for groups with followers
+  uint2* range;         // [n] of the group that key i owns: the lowest batch index below i (kEmpty: none) and the
+                        // highest above it (0: none)
   uint2* followers;     // [n] (batch index, its group's owner): the keys that repeat another key of the batch
   uint32_t* pending;    // [n] owners left for the displacement pass
   uint32_t* retry;      // [n] owners a displacement pass passes on to the next
   unsigned long long* sticky;  // [n] (batch index << 32 | bucket): buckets of timers tables whose claimed bits the
                                // finishing pass clears
   unsigned long long* fixup;   // [fix_cap] (table << 32 | bucket) whose moved counter fell to 0 off-lock
+  uint32_t n;           // keys of the batch
   uint32_t m_mask;      // m - 1 (m a power of two >= 4n)
   uint32_t idx_bits;    // bits of a batch index in a set word: n < 2^idx_bits
   uint32_t fix_cap;
@@ -101,8 +104,8 @@ cudaError_t launch_batched_lookup(const TableView* tables, uint32_t n_tables, co
                                   int keys_per_warp, bool any_timers, uint32_t blocks, unsigned long long* ctrl,
                                   cudaStream_t s);
 
-// Resets a carved workspace for a new batch: the counters to 0, the set to empty
-// (one launch).
+// Resets a carved workspace for a new batch (clear_workspace in dedup.cuh) in one
+// launch.
 cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s);
 
 // An insert call runs as a chain of kernels (the default) or as one

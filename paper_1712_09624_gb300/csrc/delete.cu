@@ -4,8 +4,8 @@
 // Kernels, in stream order, after the workspace clear:
 //   delete_kernel  per key: its owner (dedup.cuh), found in the table by the
 //                  lookup's line fetches (probe.cuh), removes the entry;
-//   delete_ranges, delete_settle  the followers before their owner in the batch:
-//                  the lowest index of each group takes over its outcome.
+//   delete_settle  the followers before their owner in the batch: the lowest
+//                  index of each group takes over its outcome.
 #include "chain_launch.h"
 #include "dedup.cuh"
 #include "probe.cuh"
@@ -100,33 +100,10 @@ __device__ __forceinline__ void settle_range(uint8_t* __restrict__ status, const
   }
 }
 
-__global__ void __launch_bounds__(kSettleThreads) delete_ranges(Workspace ws) {
-  pdl_wait();
-  pdl_release();
-  follower_ranges(ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
 __global__ void __launch_bounds__(kSettleThreads) delete_settle(uint8_t* __restrict__ status, Workspace ws) {
   pdl_wait();
   pdl_release();
   settle_range(status, ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
-// Both steps in one launch of one cluster, for batches whose followers are few
-// for its threads (13K of them: 8.6 us here, 6.7 in two launches).
-constexpr uint64_t kSettleClusterKeys = 1ull << 14;
-constexpr int kSettleClusterThreads = 1024;
-
-__global__ void __launch_bounds__(kSettleClusterThreads) delete_settle_cluster(uint8_t* __restrict__ status,
-                                                                               Workspace ws) {
-  pdl_wait();
-  pdl_release();
-  const uint32_t tid = blockIdx.x * kSettleClusterThreads + threadIdx.x, threads = gridDim.x * kSettleClusterThreads;
-  const uint32_t followers = ld32_cg(ws.counters + kCntFollowers);
-  if (!followers) return;  // the same for every block
-  follower_ranges(ws, followers, tid, threads);
-  cluster_barrier();
-  settle_range(status, ws, followers, tid, threads);
 }
 
 // A small batch in one launch of one cluster (as insert_single_launch).
@@ -146,11 +123,7 @@ __global__ void __launch_bounds__(kDeleteClusterThreads) delete_cluster(TableSet
   for (uint32_t first = blockIdx.x * kDeleteClusterThreads; first < n; first += threads)
     delete_chunk<kTM>(ts, keys, first + threadIdx.x, n, now, status, ws, stage[threadIdx.x >> 5], lists);
   cluster_barrier();
-  const uint32_t followers = ld32_cg(ws.counters + kCntFollowers);
-  if (!followers) return;  // the same for every block
-  follower_ranges(ws, followers, tid, threads);
-  cluster_barrier();
-  settle_range(status, ws, followers, tid, threads);
+  settle_range(status, ws, ld32_cg(ws.counters + kCntFollowers), tid, threads);
 }
 static_assert(kOneBlockKeys == kDeleteClusterThreads, "cluster_blocks gives batches that fit one block a cluster of one");
 
@@ -161,7 +134,7 @@ cudaError_t launch_delete(const TableSet& ts, const uint8_t* keys, uint64_t n, u
   if (n <= kClusterKeys) {
     auto kernel = !ts.any_timers ? delete_cluster<kNoTimers> : ts.views ? delete_cluster<kTimersPerKey>
                                                                        : delete_cluster<kWithTimers>;
-    return launch_cluster(kernel, false, cluster_blocks(n, kDeleteClusterThreads), kDeleteClusterThreads, 0, s, ts, keys, n, now, status,
+    return launch_cluster(kernel, cluster_blocks(n, kDeleteClusterThreads), kDeleteClusterThreads, 0, s, ts, keys, n, now, status,
                           ws);
   }
   const unsigned grid = grid_for(n, kDeleteThreads);
@@ -175,12 +148,8 @@ cudaError_t launch_delete(const TableSet& ts, const uint8_t* keys, uint64_t n, u
     e = launch_chained(delete_kernel<kTimersPerKey>, grid, kDeleteThreads, s, ts, keys, n, now, status, ws);
   }
   if (e != cudaSuccess) return e;
-  if (n <= kSettleClusterKeys)
-    return launch_cluster(delete_settle_cluster, true, kClusterMaxBlocks, kSettleClusterThreads, 0, s, status, ws);
   const unsigned most = 2u * (unsigned)device_sm_count(), want = grid_for(n, kSettleThreads);
-  const unsigned settle = want < most ? want : most;
-  if ((e = launch_chained(delete_ranges, settle, kSettleThreads, s, ws)) != cudaSuccess) return e;
-  return launch_chained(delete_settle, settle, kSettleThreads, s, status, ws);
+  return launch_chained(delete_settle, want < most ? want : most, kSettleThreads, s, status, ws);
 }
 
 }  // namespace ckpp

@@ -1072,8 +1072,6 @@ __global__ void __launch_bounds__(kThreads, 1) insert_move1(TableSet ts, const u
                                                          uint32_t* next, uint32_t* next_count) {
   pdl_wait();
   pdl_release();
-  follower_ranges(ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x,
-                  gridDim.x * blockDim.x);
   const uint32_t worker = blockIdx.x * blockDim.x + threadIdx.x, workers = gridDim.x * blockDim.x;
   const uint32_t count = ld32_cg(count_ptr);
   if (count <= min(kMoveHalfKeys, workers / 16u)) {
@@ -1263,7 +1261,7 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
   for (uint64_t j = i; j < followers; j += stride) {
     const uint2 f = ws.followers[j];
     const uint2 range = ws.range[f.y];
-    const bool last = f.x == range.y;  // its value is the one that stays
+    const bool last = f.x > f.y && f.x == range.y;  // its value is the one that stays (y of 0: none above the owner)
     // The buckets of a last occurrence are requested before the owner's outcome is looked at, both
     // at once where there are so few that the time of one counts and not their requests.
     TableView t{};
@@ -1428,10 +1426,6 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
   // retry -> last pass. A pass whose list is empty is skipped with its barrier, and so are the ones
   // after it; every block reads the same counts (final before the barrier), so all skip alike.
   Counts counts = load_counts(ws);
-  if (counts[kCntFollowers]) {
-    follower_ranges(ws, counts[kCntFollowers], tid, threads);
-    if (!counts[kCntPending]) ok &= stage_barrier<kCluster>(ws);
-  }
   if (counts[kCntPending]) {
     Node* nodes = reinterpret_cast<Node*>(smem);
     const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kSingleThreads / 32) + w;
@@ -1565,7 +1559,7 @@ cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_
       return e != cudaSuccess ? e : launch_single(ts, keys, vals, n, now, expiry, status, ws, s, per_sm);
     }
   } else if (n <= kClusterKeys) {
-    return launch_cluster(ts.any_timers ? insert_single_launch<true, true> : insert_single_launch<true, false>, false,
+    return launch_cluster(ts.any_timers ? insert_single_launch<true, true> : insert_single_launch<true, false>,
                           cluster_blocks(n, kSingleThreads), kSingleThreads, kSingleSmem, s, ts, keys, vals, n, now,
                           expiry, status, ws);
   }
