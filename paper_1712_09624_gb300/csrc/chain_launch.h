@@ -1,8 +1,12 @@
 // Host side of a call that runs as a chain of kernels on one stream (insert,
-// delete): each kernel after the first is launched with programmatic stream
-// serialization and waits for its predecessor in its first instruction
-// (pdl_wait in mutate.cuh), so that the GPU schedules it while the predecessor
-// drains.
+// delete): each kernel is launched with programmatic stream serialization and
+// waits for its predecessor in its first instruction (pdl_wait in mutate.cuh), so
+// that the GPU schedules it while the predecessor drains. That includes the
+// chain's first, the workspace clear, whose predecessor is whatever the stream
+// holds: 2 us less per call than a clear launched without (delete of 4K absent
+// keys 10.4 -> 8.6 us). It releases its successor only after its own wait, so a
+// call's other kernels start when all that was queued before the call is
+// complete, and may read the batch through the read-only path.
 #pragma once
 
 #include <cstdint>

@@ -1476,6 +1476,7 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
 
 // ------------------------------------------------------- workspace reset
 __global__ void __launch_bounds__(kThreads) workspace_clear(Workspace ws) {
+  pdl_wait();
   pdl_release();
   clear_workspace(ws, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads);
 }
@@ -1488,8 +1489,7 @@ cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s) {
   const uint64_t want = n_vec > kCounterWords ? n_vec : kCounterWords;
   const uint64_t blocks = (want + kThreads - 1) / kThreads;
   const uint64_t cap = 16ull * device_sm_count();
-  workspace_clear<<<(unsigned)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(ws);
-  return cudaGetLastError();
+  return launch_chained(workspace_clear, (unsigned)(blocks < cap ? blocks : cap), kThreads, s, ws);
 }
 
 namespace {
