@@ -28,6 +28,7 @@
 //                    has in flight;
 //   blocks per SM of the persistent grid.
 // Every configuration runs the same method and returns the same results.
+#include "chain_launch.h"
 #include "probe.cuh"
 
 namespace ckpp {
@@ -47,7 +48,7 @@ constexpr uint32_t kMaxChunksPerDraw = 8;
 
 // The number of jobs nj (*n_jobs, clamped to max_jobs), and the exclusive prefix
 // sums of their sizes in prefix[0..nj].
-__device__ uint32_t scan_jobs(const BatchJob* __restrict__ jobs, const uint32_t* __restrict__ n_jobs,
+__device__ uint32_t scan_jobs(const BatchJob* jobs, const uint32_t* n_jobs,
                               uint32_t max_jobs, unsigned long long* prefix) {
   __shared__ unsigned long long warp_sums[kBatchThreads / 32];
   // with a job per thread at most, the sizes are requested together with the count
@@ -126,8 +127,8 @@ __device__ __forceinline__ uint32_t find_job(const unsigned long long* prefix, u
 // One warp iteration: lane l < kpw owns flat keys wbase + g * kpw + l, g < G.
 // hint: the job of the lane's last key so far (0 at the start).
 template <int G, int kTM>
-__device__ __forceinline__ void lookup_chunk(const TableView* __restrict__ tables, uint32_t n_tables,
-                                             const BatchJob* __restrict__ jobs, const unsigned long long* prefix,
+__device__ __forceinline__ void lookup_chunk(const TableView* tables, uint32_t n_tables,
+                                             const BatchJob* jobs, const unsigned long long* prefix,
                                              uint32_t nj, unsigned long long total, unsigned long long wbase,
                                              uint32_t kpw, uint32_t now, uint64_t pol, uint32_t& hint,
                                              WarpStage<G>& S) {
@@ -151,7 +152,7 @@ __device__ __forceinline__ void lookup_chunk(const TableView* __restrict__ table
     if (act[g]) {
       local[g] = idx - prefix[jobi[g]];
       tv = tables[jobs[jobi[g]].table];
-      k = ld_key_ro(jobs[jobi[g]].keys + 16 * local[g], pol);
+      k = ld_key_stream(jobs[jobi[g]].keys + 16 * local[g], pol);
     }
     probe_init(p[g], k, tv.buckets, tv.nb, tv.seed, tv.timers);
   }
@@ -178,15 +179,16 @@ size_t batched_smem(uint32_t max_jobs) {
 
 // kTM: kNoTimers when no table of the batch has timers, else kTimersPerKey.
 template <int G, int kTM>
-__global__ void __launch_bounds__(kBatchThreads) batched_lookup_kernel(const TableView* __restrict__ tables,
+__global__ void __launch_bounds__(kBatchThreads) batched_lookup_kernel(const TableView* tables,
                                                                        uint32_t n_tables,
-                                                                       const BatchJob* __restrict__ jobs,
-                                                                       const uint32_t* __restrict__ n_jobs_ptr,
+                                                                       const BatchJob* jobs,
+                                                                       const uint32_t* n_jobs_ptr,
                                                                        uint32_t max_jobs, uint32_t now, uint32_t kpw,
-                                                                       unsigned long long* __restrict__ ctrl) {
+                                                                       unsigned long long* ctrl) {
   extern __shared__ __align__(128) unsigned long long prefix[];
   WarpStage<G>* stages =
       reinterpret_cast<WarpStage<G>*>(reinterpret_cast<uint8_t*>(prefix) + stage_offset(max_jobs));
+  pdl_wait();
   const uint32_t nj = scan_jobs(jobs, n_jobs_ptr, max_jobs, prefix);
   const unsigned long long total = prefix[nj];
   const uint64_t pol = policy_evict_first();
@@ -242,9 +244,8 @@ template <int G, int kTM>
 cudaError_t launch_g(const TableView* tables, uint32_t n_tables, const BatchJob* jobs, const uint32_t* n_jobs,
                      uint32_t max_jobs, uint32_t now, uint32_t kpw, uint32_t blocks, unsigned long long* ctrl,
                      cudaStream_t s) {
-  batched_lookup_kernel<G, kTM><<<blocks, kBatchThreads, batched_smem<G>(max_jobs), s>>>(
-      tables, n_tables, jobs, n_jobs, max_jobs, now, kpw, ctrl);
-  return cudaGetLastError();
+  return launch_chained_smem(batched_lookup_kernel<G, kTM>, blocks, kBatchThreads, batched_smem<G>(max_jobs), s, tables,
+                             n_tables, jobs, n_jobs, max_jobs, now, kpw, ctrl);
 }
 
 }  // namespace

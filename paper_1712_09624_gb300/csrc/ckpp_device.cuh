@@ -184,6 +184,16 @@ __device__ __forceinline__ uint16_t* expiry_ptr(const TableView& t, uint32_t b, 
   return reinterpret_cast<uint16_t*>(bucket_ptr(t, b) + kExpiryOff) + s;
 }
 
+// ------------------------------------------------- place in the stream
+// Kernels of the batch calls are launched with programmatic stream
+// serialization (chain_launch.h). Each calls
+// pdl_wait() before touching memory: it returns once the predecessor grid has
+// completed and its writes are visible (for a kernel launched without the
+// attribute it returns at once). pdl_release() lets the successor be scheduled;
+// it does not let the successor past its own wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------- memory access
 // Cache policies: L2 evict_first for data read once per lookup (bucket lines
 // of a table far larger than L2, streamed keys).
@@ -193,12 +203,20 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
   return p;
 }
 
-// 128-bit read-only streaming load.
-__device__ __forceinline__ Key ld_key_ro(const void* p, uint64_t pol) {
+// Keys of a batch. (Not by the read-only path: the kernel that wrote them may
+// still have been running when the reading one was scheduled.) ld_key_stream: of
+// a batch read once.
+__device__ __forceinline__ Key ld_key(const void* p) {
   Key k;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.u64 {%0,%1}, [%2], %3;"
+  asm volatile("ld.global.v2.u64 {%0,%1}, [%2];" : "=l"(k.k0), "=l"(k.k1) : "l"(p) : "memory");
+  return k;
+}
+__device__ __forceinline__ Key ld_key_stream(const void* p, uint64_t pol) {
+  Key k;
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.u64 {%0,%1}, [%2], %3;"
                : "=l"(k.k0), "=l"(k.k1)
-               : "l"(p), "l"(pol));
+               : "l"(p), "l"(pol)
+               : "memory");
   return k;
 }
 // Coherent (L2) loads and stores for data other threads modify.

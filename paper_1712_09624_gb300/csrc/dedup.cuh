@@ -26,10 +26,12 @@ namespace ckpp {
 constexpr uint32_t kWarpAll = 0xFFFFFFFFu;
 constexpr uint32_t kNoIndex = 0xFFFFFFFFu;
 
-__device__ __forceinline__ Key load_key(const uint8_t* keys, uint64_t i) {
-  uint64_t a, b;
-  asm volatile("ld.global.nc.v2.u64 {%0,%1}, [%2];" : "=l"(a), "=l"(b) : "l"(keys + 16 * i));
-  return Key{a, b};
+__device__ __forceinline__ Key load_key(const uint8_t* keys, uint64_t i) { return ld_key(keys + 16 * i); }
+// As ld_key, not by the read-only path.
+__device__ __forceinline__ uint64_t load_val(const uint64_t* vals, uint64_t i) {
+  uint64_t v;
+  asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(vals + i) : "memory");
+  return v;
 }
 
 // The set word of batch key i (h1: its primary hash).

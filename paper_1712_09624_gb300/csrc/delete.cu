@@ -102,7 +102,6 @@ __device__ __forceinline__ void settle_range(uint8_t* __restrict__ status, const
 
 __global__ void __launch_bounds__(kSettleThreads) delete_settle(uint8_t* __restrict__ status, Workspace ws) {
   pdl_wait();
-  pdl_release();
   settle_range(status, ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
@@ -118,6 +117,7 @@ __global__ void __launch_bounds__(kDeleteClusterThreads) delete_cluster(TableSet
   const uint32_t tid = blockIdx.x * kDeleteClusterThreads + threadIdx.x, threads = gridDim.x * kDeleteClusterThreads;
   const Workspace ws = gridDim.x == 1 ? in_shared(caller_ws, one_set, one_groups) : caller_ws;
   lists_init(lists);
+  pdl_wait();
   clear_workspace(ws, tid, threads);
   cluster_barrier();
   for (uint32_t first = blockIdx.x * kDeleteClusterThreads; first < n; first += threads)

@@ -314,7 +314,7 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
     tid = ts.id(i);
     t = ts.of(i);
     k = load_key(keys, i);
-    v = vals[i];
+    v = load_val(vals, i);
     a = address_of(k, t.nb, t.seed, h1);
     probe = set_probe(ws, h1, tid, i);
   }
@@ -950,7 +950,7 @@ __device__ void move1_range(const TableSet& ts, const uint8_t* __restrict__ keys
   for (uint32_t j = worker; j < count; j += workers) {
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
-    const uint64_t v = vals[i];
+    const uint64_t v = load_val(vals, i);
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
     uint32_t x = 0, sx = 0, y = 0, hole = 0;
@@ -1031,7 +1031,7 @@ __device__ void move1_range_half(const TableSet& ts, const uint8_t* __restrict__
     uint32_t x = 0, y = 0, f = 0;
     if (act) {
       t = ts.of(i);
-      v = vals[i];
+      v = load_val(vals, i);
       k = load_key(keys, i);
       a = address_of(k, t.nb, t.seed);
       x = lane < 8u ? a.b1 : a.b2;
@@ -1099,7 +1099,7 @@ __device__ void phase2_range(const TableSet& ts, const uint8_t* __restrict__ key
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
     const uint32_t tid = ts.id(i);
-    const uint64_t v = vals[i];
+    const uint64_t v = load_val(vals, i);
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
     uint8_t st = kStFull;
@@ -1145,7 +1145,7 @@ __device__ void phase2_range_warp(const TableSet& ts, const uint8_t* __restrict_
     const uint32_t i = list[j];
     const TableView t = ts.of(i);
     const uint32_t tid = ts.id(i);
-    const uint64_t v = vals[i];
+    const uint64_t v = load_val(vals, i);
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
     uint8_t st = kStFull;
@@ -1289,8 +1289,8 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
       const int in1 = find_key(t, a.b1, (uint32_t)s1.w[3], s1, k, a.tag);
       if (in1 < 0 && !few) ld256_cg(bucket_ptr(t, a.b2), s2.w);
       const int in2 = in1 >= 0 ? -1 : find_key(t, a.b2, (uint32_t)s2.w[3], s2, k, a.tag);
-      if (in1 >= 0) st64_cg(value_ptr(t, a.b1, in1), vals[f.x]);
-      if (in2 >= 0) st64_cg(value_ptr(t, a.b2, in2), vals[f.x]);
+      if (in1 >= 0) st64_cg(value_ptr(t, a.b1, in1), load_val(vals, f.x));
+      if (in2 >= 0) st64_cg(value_ptr(t, a.b2, in2), load_val(vals, f.x));
     }
   }
 }
@@ -1299,7 +1299,6 @@ __global__ void __launch_bounds__(kThreads) insert_fixup_finish(TableSet ts, con
                                                                 const uint64_t* __restrict__ vals,
                                                                 uint8_t* __restrict__ status, Workspace ws) {
   pdl_wait();
-  pdl_release();
   fixup_finish_range(ts, keys, vals, status, ws, load_counts(ws), blockIdx.x * (uint64_t)blockDim.x + threadIdx.x,
                      (uint64_t)gridDim.x * blockDim.x);
 }
@@ -1410,6 +1409,7 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
                                        *reinterpret_cast<OneBlockGroups*>(smem + kOneGroupsAt))
                            : caller_ws;
   bool ok = true;
+  pdl_wait();
   if (kCluster) {
     clear_workspace(ws, tid, threads);
     stage_barrier<kCluster>(ws);

@@ -11,6 +11,7 @@
 // span of the batch, with their next keys prefetched, ran 10-20% slower.)
 // Keys are read with coalesced 16-byte loads and results written with
 // coalesced stores.
+#include "chain_launch.h"
 #include "probe.cuh"
 
 namespace ckpp {
@@ -22,7 +23,7 @@ constexpr int kWarpsPerBlock = kLookupThreads / 32;
 
 // kHostIO: keys and results live in pinned host memory, reached over
 // NVLink-C2C by the loads and stores themselves (no staging copy); such keys
-// are read with plain loads, without the read-only path or L2 hints, and each
+// are read with plain loads, without cache hints, and each
 // warp writes its results as 16-byte vectors (small scattered stores are what
 // the link does worst) when the output pointers allow it.
 // kCount: no results; the secondary-line, record and second-line reads are
@@ -39,15 +40,11 @@ __global__ void __launch_bounds__(kLookupThreads) lookup_kernel(TableView t, con
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t c = (uint64_t)blockIdx.x * kWarpsPerBlock + warp;  // the warp's 32-key chunk
   const uint64_t i = c * 32 + lane;
+  pdl_wait();
   bool act[1] = {i < n};
   Key k{0, 0};
   if (act[0]) {
-    if (kHostIO) {
-      const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(keys + 16 * i);
-      k = Key{kk.x, kk.y};
-    } else {
-      k = ld_key_ro(keys + 16 * i, policy_evict_first());
-    }
+    k = kHostIO ? ld_key(keys + 16 * i) : ld_key_stream(keys + 16 * i, policy_evict_first());
   }
   Probe p[1];
   probe_init(p[0], k, t.buckets, t.nb, t.seed, t.timers);
@@ -103,8 +100,9 @@ __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView
                                                                        uint32_t refresh_ttl) {
   constexpr uint32_t timers = kTM == kWithTimers ? 1u : 0u;
   const uint64_t i = blockIdx.x * (uint64_t)kDirectThreads + threadIdx.x;
+  pdl_wait();
   if (i >= n) return;
-  const Key k = ld_key_ro(keys + 16 * i, policy_evict_first());
+  const Key k = ld_key_stream(keys + 16 * i, policy_evict_first());
   const uint64_t h1 = hash_key(k, t.seed);
   const uint32_t tag = (uint32_t)(h1 & 0xFFFF);
   uint32_t b = reduce(h1, t.nb);
@@ -157,27 +155,18 @@ constexpr uint64_t kDirectBytes = 256ull << 20;
 cudaError_t launch_direct(const TableView& t, const uint8_t* keys, uint64_t n, uint64_t* out_vals, uint8_t* out_found,
                           uint32_t now, uint32_t refresh_ttl, cudaStream_t s) {
   const uint64_t blocks = (n + kDirectThreads - 1) / kDirectThreads;
-  if (t.timers) {
-    lookup_direct_kernel<kWithTimers>
-        <<<(unsigned)blocks, kDirectThreads, 0, s>>>(t, keys, n, out_vals, out_found, now, refresh_ttl);
-  } else {
-    lookup_direct_kernel<kNoTimers><<<(unsigned)blocks, kDirectThreads, 0, s>>>(t, keys, n, out_vals, out_found, now, 0u);
-  }
-  return cudaGetLastError();
+  return launch_chained(t.timers ? lookup_direct_kernel<kWithTimers> : lookup_direct_kernel<kNoTimers>, (unsigned)blocks,
+                        kDirectThreads, s, t, keys, n, out_vals, out_found, now, t.timers ? refresh_ttl : 0u);
 }
 
 template <bool kCount, bool kHostIO, int kVariant>
 cudaError_t launch(const TableView& t, const uint8_t* keys, uint64_t n, uint64_t* out_vals, uint8_t* out_found,
                    uint32_t now, uint32_t refresh_ttl, unsigned long long* counts, cudaStream_t s) {
   const uint64_t blocks = ((n + 31) / 32 + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  if (t.timers) {
-    lookup_kernel<kCount, kHostIO, kVariant, kWithTimers><<<(unsigned)blocks, kLookupThreads, 0, s>>>(
-        t, keys, n, out_vals, out_found, now, refresh_ttl, counts);
-  } else {
-    lookup_kernel<kCount, kHostIO, kVariant, kNoTimers><<<(unsigned)blocks, kLookupThreads, 0, s>>>(
-        t, keys, n, out_vals, out_found, now, 0u, counts);
-  }
-  return cudaGetLastError();
+  return launch_chained(t.timers ? lookup_kernel<kCount, kHostIO, kVariant, kWithTimers>
+                                 : lookup_kernel<kCount, kHostIO, kVariant, kNoTimers>,
+                        (unsigned)blocks, kLookupThreads, s, t, keys, n, out_vals, out_found, now,
+                        t.timers ? refresh_ttl : 0u, counts);
 }
 
 }  // namespace
