@@ -6,10 +6,11 @@
 // in a 32 MB table 18.5 -> 16.1 us, of 50K in a 1 GB table 6.3 -> 4.5, a batched
 // launch of 48 jobs 8.3 -> 6.0, insert and delete of one key 12.5 -> 8.8, delete
 // of 4K absent keys 10.4 -> 8.1.
-// The last kernel of a call does not release its successor early: blocks of the
-// next call's first kernel that become resident beside a lookup's run, and its
-// successors after it, with the lookup's split of L1 and shared memory (a
-// million keys inserted, looked up and deleted: 375 us instead of 342).
+// No kernel releases its successor before its own end: blocks of a kernel that
+// become resident beside another's keep that one's split of L1 and shared memory,
+// and hand it on to the kernels after them (a million keys inserted, looked up
+// and deleted: 375 us with early releases everywhere, 342 without any in a call's
+// last kernel, 336 without any).
 #pragma once
 
 #include <cstdint>
@@ -41,10 +42,10 @@ cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned bl
 }
 
 // Batches this small run as one launch of one cluster, without a chain. Insert
-// and delete of n keys (with the first kernels launched plainly), back to back through the C ABI, 2^17 buckets at load
-// 0.8, a tenth of the keys repeated, chain / cluster in us: 1 key 20.5 / 12.5,
-// 64 29.1 / 20.1, 256 29.8 / 22.7, 1024 36.1 / 28.8, 2048 43.2 / 35.1, 3072 42.4
-// / 47.1: beyond 2048 keys a cluster's 2048 threads take several each.
+// and delete of n keys, back to back through the C ABI, 2^17 buckets at load
+// 0.8, a tenth of the keys repeated, chain / cluster in us: 768 keys 30.9 /
+// 24.3, 1024 31.0 / 24.1, 1536 34.9 / 28.0, 2048 35.9 / 29.0, 3072 34.4 / 38.3,
+// 4096 34.9 / 39.9: beyond 2048 keys a cluster's 2048 threads take several each.
 constexpr uint64_t kClusterKeys = 2048;
 constexpr unsigned kClusterMaxBlocks = 8;  // the portable cluster size
 

@@ -186,13 +186,10 @@ __device__ __forceinline__ uint16_t* expiry_ptr(const TableView& t, uint32_t b, 
 
 // ------------------------------------------------- place in the stream
 // Kernels of the batch calls are launched with programmatic stream
-// serialization (chain_launch.h). Each calls
-// pdl_wait() before touching memory: it returns once the predecessor grid has
-// completed and its writes are visible (for a kernel launched without the
-// attribute it returns at once). pdl_release() lets the successor be scheduled;
-// it does not let the successor past its own wait.
+// serialization (chain_launch.h). Each calls pdl_wait() before touching memory:
+// it returns once the predecessor grid has completed and its writes are visible
+// (for a kernel launched without the attribute it returns at once).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------- memory access
 // Cache policies: L2 evict_first for data read once per lookup (bucket lines

@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(kDeleteThreads) delete_kernel(TableSet ts, con
   __shared__ BlockLists<1> lists;
   lists_init(lists);
   pdl_wait();
-  pdl_release();
   delete_chunk<kTM>(ts, keys, blockIdx.x * (uint64_t)kDeleteThreads + threadIdx.x, n, now, status, ws,
                     stage[threadIdx.x >> 5], lists);
 }

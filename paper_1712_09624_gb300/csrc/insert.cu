@@ -415,7 +415,6 @@ __global__ void __launch_bounds__(kP1Threads, 1024 / kP1Threads) insert_phase1(T
   __shared__ P1Lists lists;
   lists_init(lists);
   pdl_wait();
-  pdl_release();
   const uint64_t i = blockIdx.x * (uint64_t)kP1Threads + threadIdx.x;
   phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
 }
@@ -1071,7 +1070,6 @@ __global__ void __launch_bounds__(kThreads, 1) insert_move1(TableSet ts, const u
                                                          const uint32_t* list, const uint32_t* count_ptr,
                                                          uint32_t* next, uint32_t* next_count) {
   pdl_wait();
-  pdl_release();
   const uint32_t worker = blockIdx.x * blockDim.x + threadIdx.x, workers = gridDim.x * blockDim.x;
   const uint32_t count = ld32_cg(count_ptr);
   if (count <= min(kMoveHalfKeys, workers / 16u)) {
@@ -1184,7 +1182,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) insert_phase2_warp(TableSet ts
                                                                   const uint32_t* count_ptr, uint32_t* retry,
                                                                   uint32_t* retry_count, uint32_t max_keys) {
   pdl_wait();
-  pdl_release();
   static_assert(kWarps * warp_search_bytes<kBfsNodes>() <= 48 * 1024, "search state exceeds 48 KB");
   __shared__ Node queues[kWarps][kBfsNodes];
   __shared__ uint32_t sets[kWarps][WarpSeen<kBfsNodes>::kSize];
@@ -1202,7 +1199,6 @@ __global__ void __launch_bounds__(kThreadsPerBlock) insert_phase2(TableSet ts, c
                                                                   const uint32_t* count_ptr, uint32_t* retry,
                                                                   uint32_t* retry_count, uint32_t max_keys) {
   pdl_wait();
-  pdl_release();
   static_assert(kThreadsPerBlock * kBfsNodes * sizeof(Node) <= 48 * 1024, "BFS state exceeds 48 KB");
   static_assert(kThreadsPerBlock % 32 == 0 &&
                     (kThreadsPerBlock / 32) * warp_search_bytes<kBfsNodes>() <= kBfsNodes * kThreadsPerBlock * sizeof(Node),
@@ -1477,7 +1473,6 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
 // ------------------------------------------------------- workspace reset
 __global__ void __launch_bounds__(kThreads) workspace_clear(Workspace ws) {
   pdl_wait();
-  pdl_release();
   clear_workspace(ws, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads);
 }
 
