@@ -90,8 +90,9 @@ __global__ void __launch_bounds__(kLookupThreads) lookup_kernel(TableView t, con
 // of its own, which is why lookup_kernel fetches whole lines; in L2 they run at
 // 250 G/s, and lookup_kernel is bound by its 22 warp instructions per lookup
 // instead. 1M keys, half of them unknown, load 0.9: 26.8 -> 14.4 us on a 32 MB
-// table (28.8 -> 18.8 when three such tables take turns).
-constexpr int kDirectThreads = 256;
+// table (28.8 -> 18.8 when three such tables take turns, 16.1 since calls are
+// chained). Blocks of 128 threads: 15.7, of 64 and 256 16.1, of 512 16.7.
+constexpr int kDirectThreads = 128;
 
 template <int kTM>
 __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView t, const uint8_t* __restrict__ keys,
