@@ -1256,17 +1256,17 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
   const bool few = followers <= 16384u;
   for (uint64_t j = i; j < followers; j += stride) {
     const uint2 f = ws.followers[j];
+    const Key k = load_key(keys, f.x);
+    const uint64_t v = load_val(vals, f.x);
     const uint2 range = ws.range[f.y];
     const bool last = f.x > f.y && f.x == range.y;  // its value is the one that stays (y of 0: none above the owner)
     // The buckets of a last occurrence are requested before the owner's outcome is looked at, both
     // at once where there are so few that the time of one counts and not their requests.
     TableView t{};
-    Key k{0, 0};
     Addr a{};
     Snap s1{}, s2{};
     if (last) {
       t = ts.of(f.x);
-      k = load_key(keys, f.x);
       a = address_of(k, t.nb, t.seed);
       ld256_cg(bucket_ptr(t, a.b1), s1.w);
       if (few) ld256_cg(bucket_ptr(t, a.b2), s2.w);
@@ -1285,8 +1285,8 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
       const int in1 = find_key(t, a.b1, (uint32_t)s1.w[3], s1, k, a.tag);
       if (in1 < 0 && !few) ld256_cg(bucket_ptr(t, a.b2), s2.w);
       const int in2 = in1 >= 0 ? -1 : find_key(t, a.b2, (uint32_t)s2.w[3], s2, k, a.tag);
-      if (in1 >= 0) st64_cg(value_ptr(t, a.b1, in1), load_val(vals, f.x));
-      if (in2 >= 0) st64_cg(value_ptr(t, a.b2, in2), load_val(vals, f.x));
+      if (in1 >= 0) st64_cg(value_ptr(t, a.b1, in1), v);
+      if (in2 >= 0) st64_cg(value_ptr(t, a.b2, in2), v);
     }
   }
 }
