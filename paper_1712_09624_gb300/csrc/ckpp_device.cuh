@@ -216,6 +216,7 @@ __device__ __forceinline__ Key ld_key_stream(const void* p, uint64_t pol) {
                : "memory");
   return k;
 }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // Coherent (L2) loads and stores for data other threads modify.
 __device__ __forceinline__ void ld256_cg(const void* p, uint64_t (&w)[4]) {
   asm volatile("ld.global.relaxed.gpu.v4.u64 {%0,%1,%2,%3}, [%4];"
