@@ -14,7 +14,7 @@ namespace ckpp {
 
 namespace {
 
-constexpr int kDeleteThreads = 128;
+constexpr int kDeleteThreads = 64;  // 1M absent keys: 55.9 us, with 128 56.9, with 32 58.6
 constexpr int kDeleteClusterThreads = 256;
 constexpr int kSettleThreads = 256;
 
