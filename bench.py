@@ -577,7 +577,6 @@ def small_config(args, dev, stream, steps: int = 200, warmup: int = 5):
                          "frac": round(b / per / 1e9 / l2, 4),
                          "peak_kind": "measured L2 streaming read (ckpp_wl_l2_read, 48 MiB buffer, 20 passes, "
                                       "best of 10 launches)",
-                         "whole_lines_frac": round(line_bytes_of(c, n) / per / 1e9 / l2, 4),
                          "frac_of_hbm_copy": round(b / per / 1e9 / hbm, 4)}}
 
 
@@ -654,6 +653,9 @@ def mutation_rates(table, dev, stream, ins_times, seed):
     fill_keys = W.make_keys(seed, W.STREAM_INSERT_KEYS, 1 << 20)
     k = torch.from_numpy(fill_keys).to(dev)
     vals = torch.arange(k.shape[0], dtype=torch.int64, device=dev)
+    for _ in range(3):  # untimed: the first calls of a process load their kernels on the host
+        table.delete(k, 0, stream)
+        table.insert(k, vals, 0, 0, stream)
     torch.cuda.synchronize()
     e = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
     e[0].record(stream)
