@@ -278,8 +278,8 @@ int ckpp_bulk_insert(ckpp_table* table, const ckpp_key* keys, const uint64_t* va
  *   CKPP_INSERT_LAUNCH_CHAIN   (the default) a chain of dependent kernels:
  *                              duplicate resolution and the slot claims, the
  *                              one-move pass, three cuckoo-path searches, the
- *                              filter fixup, each launched to start while its
- *                              predecessor drains; a batch of at most 2048
+ *                              filter fixup, the launch of each prepared while
+ *                              its predecessor runs; a batch of at most 2048
  *                              keys runs the same stages in one launch of one
  *                              thread-block cluster;
  *   CKPP_INSERT_LAUNCH_SINGLE  one cooperative launch running the same stages

@@ -31,9 +31,8 @@
 //             outcome, later ones UPDATED, or FULL/BUSY; the last one's value
 //             is stored), which gives the batch the result of inserting its
 //             keys one by one in index order.
-// Before them, one kernel clears the workspace (counters and the set). Each
-// kernel after it waits for its predecessor in its first instruction
-// (chain_launch.h).
+// Before them, one kernel clears the workspace (counters, set and ranges). Each
+// kernel waits for its predecessor in its first instruction (chain_launch.h).
 #include "chain_launch.h"
 #include "dedup.cuh"
 
