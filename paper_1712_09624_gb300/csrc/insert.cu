@@ -120,6 +120,14 @@ struct P1Bucket {
   uint64_t bloom;
 };
 
+// Which of r's slots are dead and which carry the batch's own expiry, from one
+// reading of the expiries (e0, e1): another key's expiry that makes a dead slot
+// look alive always shows in fresh as well.
+__device__ __forceinline__ void p1_expiries(P1Bucket& r, uint64_t e0, uint64_t e1, uint32_t now, uint32_t expiry) {
+  r.dead = r.ctrl & ~alive_mask(e0, e1, now) & kBusyMask;
+  r.fresh = r.match ? tag_mask(e0, e1, expiry) : 0u;
+}
+
 __device__ __forceinline__ P1Bucket p1_bucket(const TableView& t, uint32_t b, const Snap& s, uint32_t tag, bool timers,
                                               uint32_t now, uint32_t expiry) {
   P1Bucket r;
@@ -129,13 +137,12 @@ __device__ __forceinline__ P1Bucket p1_bucket(const TableView& t, uint32_t b, co
   r.bloom = s.w[2];
   r.dead = r.fresh = 0;
   if (timers) {
-    if (r.match) r.fresh = tag_mask(s.e0, s.e1, expiry);
-    r.dead = r.ctrl & ~alive_mask(s.e0, s.e1, now) & kBusyMask;
+    p1_expiries(r, s.e0, s.e1, now, expiry);
     if (r.dead) {  // read again behind the ctrl word
       fence_acq_rel();
       uint64_t e0, e1;
       ld128_cg(expiry_ptr(t, b, 0), e0, e1);
-      r.dead = r.ctrl & ~alive_mask(e0, e1, now) & kBusyMask;
+      p1_expiries(r, e0, e1, now, expiry);
     }
   }
   return r;
