@@ -178,9 +178,11 @@ __device__ __forceinline__ void clear_workspace(const Workspace& ws, uint32_t wo
 }
 
 // All threads of the cluster arrive; what each wrote before is seen by all after.
+// Not the .aligned forms: those want every warp whole at the barrier, and lanes
+// come to it from loops and lock waits of different lengths.
 __device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 }  // namespace ckpp
