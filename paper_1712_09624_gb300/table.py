@@ -61,6 +61,8 @@ class FlowTable:
         k = as_device_keys(keys, self.device)
         v = as_device_values(values, self.device)
         n = k.shape[0]
+        if v.numel() < n:
+            raise ValueError(f"{v.numel()} values for {n} keys")
         status = torch.empty(n, dtype=torch.uint8, device=self.device)
         K.table_insert(self.handle, k, v, status, self.workspace(n), now, ttl, stream)
         return status
