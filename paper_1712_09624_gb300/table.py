@@ -54,7 +54,8 @@ class FlowTable:
             need = K.ckpp_workspace_bytes(n)
             if self._ws is None or self._ws.numel() < need:
                 self._ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-            self._ws_keys = n  # a smaller batch never needs more
+            if need:  # 0: more keys than a batch can have, which the call reports
+                self._ws_keys = n  # a smaller batch never needs more
         return self._ws
 
     def insert(self, keys, values, now: int = 0, ttl: int = 0, stream=None) -> torch.Tensor:

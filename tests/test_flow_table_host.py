@@ -29,3 +29,11 @@ def test_insert_refuses_fewer_values_than_keys(table, monkeypatch, n, values, as
         assert calls == []
     else:
         assert table.insert(k, v).shape == (n,) and calls == [(n, values)]
+
+
+@pytest.mark.parametrize("first", [0, 100, (1 << 30) + 1])
+def test_workspace_suits_every_batch_after_one_that_is_too_large(table, first):
+    table.workspace(first)
+    table.workspace((1 << 30) + 1)
+    for n in (1, 99, 5000, 200):
+        assert table.workspace(n).numel() >= K.ckpp_workspace_bytes(n) > 0, n
