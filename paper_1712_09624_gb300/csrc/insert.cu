@@ -202,7 +202,7 @@ __device__ __forceinline__ int p1_find(const TableView& t, const P1Bucket& r, co
 
 // Claim the slot of the key's own dead entry (slot sl of bucket b, busy in c).
 // Returns 1 on success, 0 if another key took the slot first (the entry is
-// gone), -2 after kClaimAttempts failed CASes.
+// gone), -2 (latched) after kClaimAttempts failed CASes.
 __device__ int claim_revival(const TableView& t, uint32_t b, uint32_t sl, uint32_t c) {
   uint32_t* cp = ctrl_ptr(t, b);
   for (int i = 0; i < kClaimAttempts; ++i) {
@@ -211,6 +211,7 @@ __device__ int claim_revival(const TableView& t, uint32_t b, uint32_t sl, uint32
     if (got == c) return 1;
     c = got;
   }
+  latch_error(t, kErrLockTimeout);
   return -2;
 }
 
@@ -244,7 +245,7 @@ __device__ __forceinline__ uint8_t p1_stored(const TableView& t, const P1Bucket&
 }
 
 // Claim the lowest claimable slot of bucket r. Returns the slot (prev receives
-// the word the CAS replaced), -1 if nothing is claimable, -2 after
+// the word the CAS replaced), -1 if nothing is claimable, -2 (latched) after
 // kClaimAttempts failed CASes.
 __device__ __forceinline__ int claim_slot(const TableView& t, const P1Bucket& r, uint32_t& prev) {
   uint32_t* cp = ctrl_ptr(t, r.b);
@@ -261,6 +262,7 @@ __device__ __forceinline__ int claim_slot(const TableView& t, const P1Bucket& r,
     }
     c = got;
   }
+  latch_error(t, kErrLockTimeout);
   return -2;
 }
 
@@ -370,7 +372,6 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
         }
         if (sl == -2) {
           st = kStBusy;
-          latch_error(t, kErrLockTimeout);
           break;
         }
         if (r.b == a.b2) break;

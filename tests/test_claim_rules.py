@@ -12,10 +12,11 @@ import host_model as H
 
 # Memory accesses of the model. Time passes with every access of the key that is
 # watched. The other key's claim, its entry's key and expiry, and its publication
-# become visible at times of their own (ev[0..3]).
+# become visible at times of their own (ev[0..3]); cas_fails: every CAS finds its
+# word changed.
 ACCESS = """
 static uint8_t bucket_mem[256];
-static int clock_now, ev[4];
+static int clock_now, ev[4], cas_fails, latched;
 static uint32_t ctrl0, slot, expiry_of_batch;
 static uint64_t other_key[2];
 static void tick();
@@ -27,11 +28,13 @@ static void ld128_cg(const void* p, uint64_t& a, uint64_t& b) {
 static uint32_t ld32_cg(const void* p) { tick(); return *(const uint32_t*)p; }
 static uint32_t atomicCAS(uint32_t* p, uint32_t want, uint32_t to) {
   tick();
+  if (cas_fails) return want ^ (1u << 30);
   const uint32_t old = *p;
   if (old == want) *p = to;
   return old;
 }
 struct Snap { uint64_t w[4]; uint64_t e0, e1; };
+static void latch_error(const TableView&, uint32_t) { ++latched; }
 """
 
 DRIVER = """
@@ -52,7 +55,7 @@ static void tick() {
 static void start(uint32_t busy, uint32_t expiry, const int* at) {
   for (int i = 0; i < 256; ++i) bucket_mem[i] = 0;
   *(uint32_t*)(bucket_mem + 24) = busy;
-  clock_now = 0;
+  clock_now = cas_fails = latched = 0;
   expiry_of_batch = expiry;
   other_key[0] = 77, other_key[1] = 78;
   for (int i = 0; i < 4; ++i) ev[i] = at[i];
@@ -85,10 +88,23 @@ extern "C" int stored(uint32_t mine, uint32_t taken, uint32_t stored_expiry, uin
   const int st = sl < 0 ? -1 : p1_stored(t, r, (uint32_t)sl, true, work);
   return st;
 }
+extern "C" int lost_claim(int revival) {
+  const int never[4] = {-1, -1, -1, -1};
+  start(revival ? 1u : 0u, 0, never);
+  cas_fails = 1;
+  P1Bucket r{};
+  r.ctrl = revival ? 1u : 0u;
+  r.dead = r.ctrl;
+  P1Work work = kP1None;
+  uint32_t prev = 0;
+  const TableView t = view();
+  const int got = revival ? p1_stored(t, r, 0, true, work) : claim_slot(t, r, prev);
+  return latched == 1 ? got : 1000 + latched;
+}
 """
 
 NOW, EXPIRY = 1000, 1040
-INSERTED, UPDATED = 1, 2
+INSERTED, UPDATED, BUSY = 1, 2, 6
 
 
 @pytest.fixture(scope="module")
@@ -124,3 +140,8 @@ def test_a_live_entry_is_updated_in_place_whatever_the_rest_of_its_bucket_does(m
     for at in schedules():
         for mine, taken in ((0, 5), (5, 0), (2, 3)):
             assert outcome(model, mine, taken, expiry, expiries_first, at) == UPDATED, at
+
+
+def test_a_claim_that_gives_up_latches_the_error(model):
+    assert model.lost_claim(1) == BUSY
+    assert model.lost_claim(0) == -2
