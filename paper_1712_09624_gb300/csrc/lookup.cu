@@ -97,8 +97,7 @@ constexpr int kDirectThreads = 128;
 template <int kTM>
 __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView t, const uint8_t* __restrict__ keys,
                                                                        uint64_t n, uint64_t* __restrict__ out_vals,
-                                                                       uint8_t* __restrict__ out_found, uint32_t now,
-                                                                       uint32_t refresh_ttl) {
+                                                                       uint8_t* __restrict__ out_found, uint32_t now) {
   constexpr uint32_t timers = kTM == kWithTimers ? 1u : 0u;
   const uint64_t i = blockIdx.x * (uint64_t)kDirectThreads + threadIdx.x;
   pdl_wait();
@@ -128,7 +127,6 @@ __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView
         if (!timers || alive16(e, now)) {  // Sec. 4.2: a dead entry is not returned
           found = true;
           value = v;
-          if (timers && refresh_ttl) set_expiry(t, b, s, now + refresh_ttl);
         }
         break;
       }
@@ -154,10 +152,10 @@ __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView
 constexpr uint64_t kDirectBytes = 256ull << 20;
 
 cudaError_t launch_direct(const TableView& t, const uint8_t* keys, uint64_t n, uint64_t* out_vals, uint8_t* out_found,
-                          uint32_t now, uint32_t refresh_ttl, cudaStream_t s) {
+                          uint32_t now, cudaStream_t s) {
   const uint64_t blocks = (n + kDirectThreads - 1) / kDirectThreads;
   return launch_chained(t.timers ? lookup_direct_kernel<kWithTimers> : lookup_direct_kernel<kNoTimers>, (unsigned)blocks,
-                        kDirectThreads, s, t, keys, n, out_vals, out_found, now, t.timers ? refresh_ttl : 0u);
+                        kDirectThreads, s, t, keys, n, out_vals, out_found, now);
 }
 
 template <bool kCount, bool kHostIO, int kVariant>
@@ -180,7 +178,7 @@ cudaError_t launch_lookup(const TableView& t, const uint8_t* keys, uint64_t n, u
     return launch<false, true, kBloom>(t, keys, n, out_vals, out_found, now, refresh_ttl, nullptr, s);
   }
   if (variant == kBloom && !refresh_ttl && t.nb * kBucketBytes <= kDirectBytes)
-    return launch_direct(t, keys, n, out_vals, out_found, now, refresh_ttl, s);
+    return launch_direct(t, keys, n, out_vals, out_found, now, s);
   switch (variant) {
     case kBloom: return launch<false, false, kBloom>(t, keys, n, out_vals, out_found, now, refresh_ttl, nullptr, s);
     case kOptimistic:

@@ -173,20 +173,6 @@ struct Snap {
   uint64_t e0, e1;
 };
 
-__device__ __forceinline__ void snap_bucket(const TableView& t, uint32_t b, Snap& s) {
-  ld256_cg(bucket_ptr(t, b), s.w);
-  if (t.timers) {
-    ld128_cg(expiry_ptr(t, b, 0), s.e0, s.e1);
-  } else {
-    s.e0 = s.e1 = 0;
-  }
-}
-
-__device__ __forceinline__ uint32_t snap_expiry(const Snap& s, uint32_t slot) {
-  const uint64_t e = slot < 4 ? s.e0 : s.e1;
-  return (uint32_t)(e >> (16 * (slot & 3))) & 0xFFFFu;
-}
-
 // Slots an insertion may take: empty, or busy with a dead entry (Sec. 4.2).
 __device__ __forceinline__ uint32_t free_mask(const TableView& t, uint32_t ctrl, const Snap& s, uint32_t now) {
   const uint32_t busy = ctrl & kBusyMask;
