@@ -57,22 +57,23 @@ constexpr uint32_t kMoveGroup = 2;
 // claimable slot of its primary, else of its secondary (Sec. 2), else waits
 // for the displacement passes.
 //
-// A claim is a CAS on the bucket's ctrl word that sets the slot's claimed bit
-// (and clears its busy and in_secondary bits: a dead entry held there is
-// evicted, with moved-counter upkeep on its own primary). A failed CAS returns
-// the current word, and the claimable slots are recomputed from it. The owner
-// then writes the entry, and after a fence one atomic XOR turns the claimed
-// bit into busy: readers look at busy slots only, and one that meets a busy
-// slot with its key's tag reads the slot's key behind a fence of its own, so
-// it never sees the bytes that a freshly published slot held before.
+// A claim is a CAS on the bucket's ctrl word that sets the slot's claimed bit.
+// A failed CAS returns the current word, and the claimable slots are recomputed
+// from it. The owner then writes the entry. A slot that was free is published
+// after a fence by one atomic XOR, which turns the claimed bit into busy:
+// readers look at busy slots only, and one that meets a busy slot with its
+// key's tag reads the slot's key behind a fence of its own, so it never sees
+// the bytes that a freshly published slot held before.
 //
-// With timers two more rules keep a slot from being taken twice. A slot counts
-// as dead only if its expiry was read after (a fence) the ctrl word that
-// showed it busy; and a slot that held a dead entry keeps its claimed bit when
-// it is published (listed in ws.sticky, cleared by the finishing pass), since
-// its ctrl word would otherwise read as it did before the claim. Reviving a
-// key's own dead entry claims its slot in the same way (busy stays set), so a
-// revival and a reuse of that slot by another key cannot both succeed.
+// A slot that holds a dead entry (timers) stays busy when it is claimed (the
+// dead entry is evicted, with moved-counter upkeep on its own primary; the
+// in_secondary bit becomes the new entry's) and keeps its claimed bit until the
+// finishing pass (listed in ws.sticky): it needs no publication, readers pass
+// over claimed slots, and its word never reads again as it did before the
+// claim. Reviving a key's own dead entry claims its slot in the same way, so a
+// revival and a reuse of that slot by another key cannot both succeed. And a
+// slot counts as dead only if its expiry was read after (a fence) the ctrl word
+// that showed it busy.
 //
 // Storing a key in its secondary sets its two bits in the primary's filter and
 // counts it in the primary's moved counter, with relaxed atomics: no filter is
@@ -114,7 +115,7 @@ __device__ __forceinline__ uint4& row_chunk(P1Rows& R, uint32_t r, uint32_t c) {
 
 // A bucket as phase 1 sees it.
 struct P1Bucket {
-  uint32_t b, ctrl, match;  // match: busy slots with the key's tag
+  uint32_t b, ctrl, match;  // match: busy slots with the key's tag that no key has claimed
   uint32_t dead;            // busy slots with a dead entry (timers)
   uint32_t fresh;           // slots with the expiry that this batch writes (timers; only where match is set)
   uint64_t bloom;
@@ -133,7 +134,7 @@ __device__ __forceinline__ P1Bucket p1_bucket(const TableView& t, uint32_t b, co
   P1Bucket r;
   r.b = b;
   r.ctrl = (uint32_t)s.w[3];
-  r.match = tag_mask(s.w[0], s.w[1], tag) & r.ctrl & kBusyMask;
+  r.match = tag_mask(s.w[0], s.w[1], tag) & r.ctrl & ~(r.ctrl >> kClaimShift) & kBusyMask;
   r.bloom = s.w[2];
   r.dead = r.fresh = 0;
   if (timers) {
@@ -244,17 +245,18 @@ __device__ __forceinline__ uint8_t p1_stored(const TableView& t, const P1Bucket&
   return kStUpdated;
 }
 
-// Claim the lowest claimable slot of bucket r. Returns the slot (prev receives
-// the word the CAS replaced), -1 if nothing is claimable, -2 (latched) after
-// kClaimAttempts failed CASes.
-__device__ __forceinline__ int claim_slot(const TableView& t, const P1Bucket& r, uint32_t& prev) {
+// Claim the lowest claimable slot of bucket r (insec: the key's secondary).
+// Returns the slot (prev receives the word the CAS replaced), -1 if nothing is
+// claimable, -2 (latched) after kClaimAttempts failed CASes.
+__device__ __forceinline__ int claim_slot(const TableView& t, const P1Bucket& r, bool insec, uint32_t& prev) {
   uint32_t* cp = ctrl_ptr(t, r.b);
   uint32_t c = r.ctrl;
   for (int i = 0; i < kClaimAttempts; ++i) {
     const uint32_t f = claimable(c, r.dead);
     if (!f) return -1;
     const uint32_t sl = __ffs(f) - 1;
-    const uint32_t want = (c | claim_bit(sl)) & ~((1u << sl) | (1u << (kInsecShift + sl)));
+    const uint32_t in = 1u << (kInsecShift + sl);
+    const uint32_t want = ((c | claim_bit(sl)) & ~in) | (insec && ((c >> sl) & 1u) ? in : 0u);
     const uint32_t got = atomicCAS(cp, c, want);
     if (got == c) {
       prev = c;
@@ -341,7 +343,7 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
   p1_fetch<kTimers>(t, a.b2, have2, R, s);
   uint8_t st = 0;
   P1Work work = kP1None;
-  uint32_t flip = 0;  // publication: the bits of the ctrl word to flip
+  uint32_t flip = 0;  // publication of a slot that was free: the bits of the ctrl word to flip
   int sl = -1;
   bool sticky = false;
   if (mine) {
@@ -355,16 +357,14 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
       if (!claimable(r.ctrl, r.dead)) r = r2;
       for (;;) {
         uint32_t prev = 0;
-        sl = claim_slot(t, r, prev);
+        sl = claim_slot(t, r, r.b == a.b2, prev);
         if (sl >= 0) {
           work = kP1Place;
           st = kStInserted;
-          flip = 1u << sl;
-          sticky = kTimers && ((prev >> sl) & 1u);  // held a dead entry
-          if (!sticky) flip |= claim_bit(sl);
+          sticky = kTimers && ((prev >> sl) & 1u);  // holds a dead entry
+          if (!sticky) flip = claim_bit(sl) | 1u << sl | (r.b == a.b2 ? 1u << (kInsecShift + sl) : 0u);
           if (sticky && ((prev >> (kInsecShift + sl)) & 1u)) evict_displaced(t, tid, r.b, sl, ws);
           if (r.b == a.b2) {  // Sec. 4.1: displaced to the secondary
-            flip |= 1u << (kInsecShift + sl);
             atomicOr(reinterpret_cast<unsigned long long*>(bloom_ptr(t, a.b1)), (unsigned long long)a.bits);
             atomicAdd(moved_ptr(t, a.b1), 1u);
           }
@@ -400,7 +400,7 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
   p1_store<kTimers>(__popc(jobs), R);
   fence_acq_rel();  // every lane's stores before any busy bit
   __syncwarp();
-  if (work == kP1Place) atomicXor(ctrl_ptr(t, r.b), flip);
+  if (flip) atomicXor(ctrl_ptr(t, r.b), flip);
   sticky |= work == kP1Revive;
   const bool queued = mine && !st, follows = act && !mine;
   uint32_t at[3];

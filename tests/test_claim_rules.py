@@ -1,7 +1,8 @@
-"""What an insert does with a key's stored entry while another key of the batch
-takes a slot of the same bucket, for every order in which that key's stores can
-become visible: the entry's words lie in different lines, so nothing orders them
-before the fence that precedes the publication; only the claim comes first."""
+"""What an insert does in a bucket while another key of the batch takes a slot of
+it, for every order in which that key's stores can become visible: the entry's
+words lie in different lines, so nothing orders them; only the claim comes first,
+and the publication of a slot that was free last (a slot that held a dead entry
+stays busy, with its claim, and has none)."""
 
 import ctypes as C
 import itertools
@@ -16,7 +17,7 @@ import host_model as H
 # word changed.
 ACCESS = """
 static uint8_t bucket_mem[256];
-static int clock_now, ev[4], cas_fails, latched;
+static int clock_now, ev[4], cas_fails, latched, was_free;
 static uint32_t ctrl0, slot, expiry_of_batch;
 static uint64_t other_key[2];
 static void tick();
@@ -47,18 +48,28 @@ static void put_expiry(uint32_t s, uint32_t e) { ((uint16_t*)(bucket_mem + kExpi
 static void tick() {
   const int t = clock_now++;
   uint32_t* ctrl = (uint32_t*)(bucket_mem + 24);
-  if (t == ev[0]) *ctrl = (*ctrl | claim_bit(slot)) & ~(1u << slot);
+  if (t == ev[0]) *ctrl |= claim_bit(slot);
   if (t == ev[1]) put_key(slot, other_key[0], other_key[1]);
   if (t == ev[2]) put_expiry(slot, expiry_of_batch);
-  if (t == ev[3]) *ctrl |= 1u << slot;
+  if (t == ev[3] && was_free) *ctrl ^= claim_bit(slot) | 1u << slot;
 }
 static void start(uint32_t busy, uint32_t expiry, const int* at) {
   for (int i = 0; i < 256; ++i) bucket_mem[i] = 0;
   *(uint32_t*)(bucket_mem + 24) = busy;
-  clock_now = cas_fails = latched = 0;
+  clock_now = cas_fails = latched = was_free = 0;
   expiry_of_batch = expiry;
   other_key[0] = 77, other_key[1] = 78;
   for (int i = 0; i < 4; ++i) ev[i] = at[i];
+}
+static Snap snapshot(int expiries_first) {
+  Snap s;
+  const uint64_t* w = (const uint64_t*)bucket_mem;
+  for (int i = 0; i < 2; ++i) {
+    tick();
+    if ((i == 0) == (expiries_first != 0)) s.e0 = w[4], s.e1 = w[5];
+    else for (int j = 0; j < 4; ++j) s.w[j] = w[j];
+  }
+  return s;
 }
 // The key has an entry in slot `mine` with expiry `stored`; the other key takes slot
 // `taken`, whose entry is dead. expiries_first: which of the snapshot's reads comes first.
@@ -74,19 +85,28 @@ extern "C" int stored(uint32_t mine, uint32_t taken, uint32_t stored_expiry, uin
   put_key(mine, k.k0, k.k1);
   put_expiry(mine, stored_expiry);
   ((uint16_t*)bucket_mem)[mine] = (uint16_t)tag;
-  Snap s;
-  const uint64_t* w = (const uint64_t*)bucket_mem;
-  for (int i = 0; i < 2; ++i) {
-    tick();
-    if ((i == 0) == (expiries_first != 0)) s.e0 = w[4], s.e1 = w[5];
-    else for (int j = 0; j < 4; ++j) s.w[j] = w[j];
-  }
+  const Snap s = snapshot(expiries_first);
   const TableView t = view();
   const P1Bucket r = p1_bucket(t, 0, s, tag, true, now, expiry);
   const int sl = p1_find(t, r, k);
   P1Work work = kP1None;
   const int st = sl < 0 ? -1 : p1_stored(t, r, (uint32_t)sl, true, work);
   return st;
+}
+// The key is not stored, and slot `taken` is the only one that it could claim: free, or
+// with a dead entry. Returns whether it claimed the slot after the other key had.
+extern "C" int claimed_twice(uint32_t taken, int free, uint32_t now, uint32_t expiry, int expiries_first,
+                             const int* at) {
+  start(free ? 0xFFu & ~(1u << taken) : 0xFFu, expiry, at);
+  slot = taken;
+  was_free = free;
+  for (uint32_t s = 0; s < 8; ++s) put_expiry(s, s == taken ? now - 20 : now + 3);
+  const Snap s = snapshot(expiries_first);
+  const TableView t = view();
+  const P1Bucket r = p1_bucket(t, 0, s, 9, true, now, expiry);
+  uint32_t prev = 0;
+  const int got = claim_slot(t, r, false, prev);
+  return got >= 0 && clock_now > at[0];
 }
 extern "C" int lost_claim(int revival) {
   const int never[4] = {-1, -1, -1, -1};
@@ -98,7 +118,7 @@ extern "C" int lost_claim(int revival) {
   P1Work work = kP1None;
   uint32_t prev = 0;
   const TableView t = view();
-  const int got = revival ? p1_stored(t, r, 0, true, work) : claim_slot(t, r, prev);
+  const int got = revival ? p1_stored(t, r, 0, true, work) : claim_slot(t, r, false, prev);
   return latched == 1 ? got : 1000 + latched;
 }
 """
@@ -140,6 +160,14 @@ def test_a_live_entry_is_updated_in_place_whatever_the_rest_of_its_bucket_does(m
     for at in schedules():
         for mine, taken in ((0, 5), (5, 0), (2, 3)):
             assert outcome(model, mine, taken, expiry, expiries_first, at) == UPDATED, at
+
+
+@pytest.mark.parametrize("expiries_first", [0, 1])
+@pytest.mark.parametrize("free", [0, 1])
+def test_a_slot_is_claimed_once(model, free, expiries_first):
+    for at in schedules():
+        for slot in (0, 5):
+            assert not model.claimed_twice(slot, free, NOW, EXPIRY, expiries_first, (C.c_int * 4)(*at)), at
 
 
 def test_a_claim_that_gives_up_latches_the_error(model):
