@@ -75,7 +75,7 @@ static Snap snapshot(int expiries_first) {
 // `taken`, whose entry is dead. expiries_first: which of the snapshot's reads comes first.
 // Returns the status (0: the key has to look for a slot), or -1 if the key was not found.
 extern "C" int stored(uint32_t mine, uint32_t taken, uint32_t stored_expiry, uint32_t now, uint32_t expiry,
-                      int expiries_first, const int* at) {
+                      int expiries_first, int as_secondary, const int* at) {
   start(1u << mine | 1u << taken, expiry, at);
   slot = taken;
   const Key k{5, 6};
@@ -87,8 +87,9 @@ extern "C" int stored(uint32_t mine, uint32_t taken, uint32_t stored_expiry, uin
   ((uint16_t*)bucket_mem)[mine] = (uint16_t)tag;
   const Snap s = snapshot(expiries_first);
   const TableView t = view();
-  const P1Bucket r = p1_bucket(t, 0, s, tag, true, now, expiry);
-  const int sl = p1_find(t, r, k);
+  P1Bucket r = p1_bucket(0, s, tag, true, now, expiry), none{};
+  bool second;
+  const int sl = as_secondary ? p1_search(t, none, r, k, now, expiry, second) : p1_search(t, r, none, k, now, expiry, second);
   P1Work work = kP1None;
   const int st = sl < 0 ? -1 : p1_stored(t, r, (uint32_t)sl, true, work);
   return st;
@@ -96,14 +97,17 @@ extern "C" int stored(uint32_t mine, uint32_t taken, uint32_t stored_expiry, uin
 // The key is not stored, and slot `taken` is the only one that it could claim: free, or
 // with a dead entry. Returns whether it claimed the slot after the other key had.
 extern "C" int claimed_twice(uint32_t taken, int free, uint32_t now, uint32_t expiry, int expiries_first,
-                             const int* at) {
+                             int as_secondary, const int* at) {
   start(free ? 0xFFu & ~(1u << taken) : 0xFFu, expiry, at);
   slot = taken;
   was_free = free;
   for (uint32_t s = 0; s < 8; ++s) put_expiry(s, s == taken ? now - 20 : now + 3);
   const Snap s = snapshot(expiries_first);
   const TableView t = view();
-  const P1Bucket r = p1_bucket(t, 0, s, 9, true, now, expiry);
+  P1Bucket r = p1_bucket(0, s, 9, true, now, expiry), none{};
+  bool second;
+  if (as_secondary) p1_search(t, none, r, Key{5, 6}, now, expiry, second);
+  else p1_search(t, r, none, Key{5, 6}, now, expiry, second);
   uint32_t prev = 0;
   const int got = claim_slot(t, r, false, prev);
   return got >= 0 && clock_now > at[0];
@@ -130,7 +134,7 @@ INSERTED, UPDATED, BUSY = 1, 2, 6
 @pytest.fixture(scope="module")
 def model(tmp_path_factory):
     code = (H.layout() + ACCESS + "constexpr int kClaimAttempts = 64;\n" +
-            H.definitions("insert.cu", "claim_bit", "claimable", "P1Bucket", "p1_expiries", "p1_bucket", "p1_find", "claim_revival",
+            H.definitions("insert.cu", "claim_bit", "claimable", "P1Bucket", "p1_expiries", "p1_bucket", "p1_find", "p1_search", "claim_revival",
                           "P1Work", "p1_stored", "claim_slot") + DRIVER)
     return C.CDLL(H.build(tmp_path_factory.mktemp("claims"), code))
 
@@ -143,31 +147,34 @@ def schedules():
                 yield claim, key, expiry, publication
 
 
-def outcome(model, mine, taken, expiry, first, at):
-    return model.stored(mine, taken, expiry, NOW, EXPIRY, first, (C.c_int * 4)(*at))
+def outcome(model, mine, taken, expiry, first, secondary, at):
+    return model.stored(mine, taken, expiry, NOW, EXPIRY, first, secondary, (C.c_int * 4)(*at))
 
 
+@pytest.mark.parametrize("secondary", [0, 1])
 @pytest.mark.parametrize("expiries_first", [0, 1])
-def test_a_dead_entry_whose_slot_is_taken_is_never_updated_in_place(model, expiries_first):
+def test_a_dead_entry_whose_slot_is_taken_is_never_updated_in_place(model, expiries_first, secondary):
     for at in schedules():
         for slot in (0, 5):  # its entry in the bucket's first and second line
-            assert outcome(model, slot, slot, NOW - 20, expiries_first, at) in (-1, 0, INSERTED), at
+            assert outcome(model, slot, slot, NOW - 20, expiries_first, secondary, at) in (-1, 0, INSERTED), at
 
 
+@pytest.mark.parametrize("secondary", [0, 1])
 @pytest.mark.parametrize("expiries_first", [0, 1])
 @pytest.mark.parametrize("expiry", [NOW, EXPIRY, EXPIRY + 5])
-def test_a_live_entry_is_updated_in_place_whatever_the_rest_of_its_bucket_does(model, expiry, expiries_first):
+def test_a_live_entry_is_updated_in_place_whatever_the_rest_of_its_bucket_does(model, expiry, expiries_first, secondary):
     for at in schedules():
         for mine, taken in ((0, 5), (5, 0), (2, 3)):
-            assert outcome(model, mine, taken, expiry, expiries_first, at) == UPDATED, at
+            assert outcome(model, mine, taken, expiry, expiries_first, secondary, at) == UPDATED, at
 
 
+@pytest.mark.parametrize("secondary", [0, 1])
 @pytest.mark.parametrize("expiries_first", [0, 1])
 @pytest.mark.parametrize("free", [0, 1])
-def test_a_slot_is_claimed_once(model, free, expiries_first):
+def test_a_slot_is_claimed_once(model, free, expiries_first, secondary):
     for at in schedules():
         for slot in (0, 5):
-            assert not model.claimed_twice(slot, free, NOW, EXPIRY, expiries_first, (C.c_int * 4)(*at)), at
+            assert not model.claimed_twice(slot, free, NOW, EXPIRY, expiries_first, secondary, (C.c_int * 4)(*at)), at
 
 
 def test_a_claim_that_gives_up_latches_the_error(model):
