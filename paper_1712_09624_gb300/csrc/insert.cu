@@ -196,9 +196,9 @@ __device__ __forceinline__ int p1_find(const TableView& t, const P1Bucket& r, co
 // What has to be read behind the ctrl words of the primary r and of the
 // secondary r2 (empty if it was not read): the expiries again, where they showed
 // a dead slot, and the keys of the slots that match. Returns the slot of key k,
-// in r2 if second, or -1. One fence and one round trip serve both buckets: a
-// fence for each reading, up to four in a row, made phase 1 of 1M keys with dead
-// entries 25 us slower than the separate kernels it took the place of.
+// in r2 if second, or -1. One fence and one round trip serve both buckets (a
+// fence for each reading, up to four in a row: an insert of 1M keys of an
+// 8M-slot table full of dead entries, half of them revived, 183 -> 162 us).
 __device__ __forceinline__ int p1_search(const TableView& t, P1Bucket& r, P1Bucket& r2, const Key& k, uint32_t now,
                                          uint32_t expiry, bool& second) {
   second = false;
@@ -417,9 +417,13 @@ __device__ __forceinline__ void phase1_one(const TableSet& ts, const uint8_t* __
   }
   __syncwarp();
   p1_store<kTimers>(__popc(jobs), R);
-  fence_acq_rel();  // every lane's stores before any busy bit
-  __syncwarp();
-  if (flip) atomicXor(ctrl_ptr(t, r.b), flip);
+  // Entries in slots that were free are published. (A fence only where there are any: the call
+  // above, which has none, 162 -> 154 us; 1M updates of a 17M-slot table 99 -> 92.)
+  if (__any_sync(kWarpAll, flip != 0u)) {
+    fence_acq_rel();                       // every lane's stores before any busy bit
+    __syncwarp();
+    if (flip) atomicXor(ctrl_ptr(t, r.b), flip);
+  }
   sticky |= work == kP1Revive;
   const bool queued = mine && !st, follows = act && !mine;
   uint32_t at[3];
