@@ -143,13 +143,17 @@ __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView
   out_found[i] = found ? 1 : 0;
 }
 
-// Largest table (bytes of buckets) that lookup_direct_kernel is used for. 4M
-// keys, all known / half of them: 115 -> 105 / 106 -> 87 us at 256 MB, 121 ->
-// 141 / 109 -> 96 us at 320 MB; with three tables taking turns 119 -> 109 / 109
-// -> 90 us at 256 MB. A lookup that refreshes its hits keeps to lookup_kernel:
-// the refresh's store follows three reads of the bucket instead of one (32 MB,
-// load 0.6, all known: 30.8 us there, 35.1 here).
-constexpr uint64_t kDirectBytes = 256ull << 20;
+// Largest table (bytes of buckets) that lookup_direct_kernel is used for: one
+// whose first lines, half of it, fit in L2. Its reads are sectors of one line,
+// but each its own DRAM access once the line has gone. 4M keys, all known, load
+// 0.3 / 0.5 / 0.9, lookup_kernel -> this one in us: 240 MB 78 -> 61 / 90 -> 68 /
+// 116 -> 101 (with timers 96 -> 76 / 108 -> 83 / 137 -> 111), 248 MB 79 -> 89 /
+// 90 -> 97 / 117 -> 104, 256 MB 79 -> 100 / 90 -> 103 / 117 -> 104 (with timers
+// 96 -> 132 / 110 -> 131 / 139 -> 114). Tables that take turns, 512 MB or more
+// in all, gain as much up to 240 MB each. A lookup that refreshes its hits keeps
+// to lookup_kernel: the refresh's store follows three reads of the bucket instead
+// of one (32 MB, load 0.6, all known: 30.8 us there, 35.1 here).
+constexpr uint64_t kDirectBytes = 240ull << 20;
 
 cudaError_t launch_direct(const TableView& t, const uint8_t* keys, uint64_t n, uint64_t* out_vals, uint8_t* out_found,
                           uint32_t now, cudaStream_t s) {
