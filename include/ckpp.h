@@ -280,8 +280,9 @@ int ckpp_bulk_insert(ckpp_table* table, const ckpp_key* keys, const uint64_t* va
  *                              one-move pass, three cuckoo-path searches, the
  *                              filter fixup, the launch of each prepared while
  *                              its predecessor runs; a batch of at most 2048
- *                              keys runs the same stages in one launch of one
- *                              thread-block cluster;
+ *                              keys runs the same stages on one thread-block
+ *                              cluster, with one launch after it (for more than
+ *                              64 keys) for the searches that are left;
  *   CKPP_INSERT_LAUNCH_SINGLE  one cooperative launch running the same stages
  *                              separated by grid-wide barriers, sized to the
  *                              batch, with stages that have nothing to do

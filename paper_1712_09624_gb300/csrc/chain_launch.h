@@ -41,7 +41,8 @@ cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned bl
   return launch_chained_smem(kernel, grid, block, 0, s, args...);
 }
 
-// Batches this small run as one launch of one cluster, without a chain. Insert
+// Batches this small run on one cluster, without a chain (inserts of more than 64
+// keys with one launch after it, insert.cu, which is not in these figures). Insert
 // and delete of n keys, back to back through the C ABI, 2^17 buckets at load
 // 0.8, a tenth of the keys repeated, chain / cluster in us: 768 keys 30.9 /
 // 24.3, 1024 31.0 / 24.1, 1536 34.9 / 28.0, 2048 35.9 / 29.0, 3072 34.4 / 38.3,

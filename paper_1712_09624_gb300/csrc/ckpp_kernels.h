@@ -43,6 +43,7 @@ constexpr uint32_t kCntGrid = 5;           // keys the grid search left (in `pen
 constexpr uint32_t kCntSecond = 6;         // keys the second search left (in `retry`)
 constexpr uint32_t kCntSticky = 7;         // claimed bits to clear (in `sticky`)
 constexpr uint32_t kCntBarrier = 8;        // two words: the grid barrier of the single-launch insert
+constexpr uint32_t kCntRest = 10;          // blocks of the launch after a small batch's cluster that are done
 constexpr uint32_t kCounterWords = 64;
 
 // Device scratch for one insert or delete batch (carved out of the caller's

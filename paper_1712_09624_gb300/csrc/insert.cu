@@ -1156,6 +1156,23 @@ __device__ void phase2_range(const TableSet& ts, const uint8_t* __restrict__ key
   }
 }
 
+// One key's search by a whole warp (bfs_warp) and the execution of the path it
+// finds: INSERTED, BUSY, or FULL if there is no path within the search's bounds.
+template <int kBfsNodes, int kBfsDepth>
+__device__ uint8_t search_warp(const TableView& t, uint32_t tid, const Key& k, uint64_t v, const Addr& a, uint32_t now,
+                               uint32_t expiry, const Workspace& ws, Node* q, uint32_t* seen) {
+  static_assert(kBfsDepth <= kMaxDepth, "path longer than the lock set");
+  for (int attempt = 0; attempt < kPathAttempts; ++attempt) {
+    uint32_t hole = 0;
+    const int end = bfs_warp<kBfsNodes, kBfsDepth>(t, a, now, q, seen, hole);
+    if (end < 0) break;
+    const int r = execute_path_warp(t, tid, q, end, hole, k, v, a, now, expiry, ws);
+    __syncwarp();  // every lane is done with the queue
+    if (r != 0) return r > 0 ? kStInserted : kStBusy;
+  }
+  return kStFull;
+}
+
 // phase2_range with one warp per key (bfs_warp): warp / warps are this warp's
 // index among the warps sharing the pass; q and seen are the warp's own.
 // listed: the list's length (read by the caller after the list was final).
@@ -1165,7 +1182,6 @@ __device__ void phase2_range_warp(const TableSet& ts, const uint8_t* __restrict_
                                   uint8_t* __restrict__ status, const Workspace& ws, const uint32_t* list,
                                   uint32_t listed, uint32_t* retry, uint32_t* retry_count,
                                   uint32_t max_keys, Node* q, uint32_t* seen, uint32_t warp, uint32_t warps) {
-  static_assert(kBfsDepth <= kMaxDepth, "path longer than the lock set");
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t count = min(listed, max_keys);
   for (uint32_t j = count + warp * 32 + lane; j < listed; j += warps * 32) status[list[j]] = kStFull;
@@ -1176,18 +1192,7 @@ __device__ void phase2_range_warp(const TableSet& ts, const uint8_t* __restrict_
     const uint64_t v = load_val(vals, i);
     const Key k = load_key(keys, i);
     const Addr a = address_of(k, t.nb, t.seed);
-    uint8_t st = kStFull;
-    for (int attempt = 0; attempt < kPathAttempts; ++attempt) {
-      uint32_t hole = 0;
-      const int end = bfs_warp<kBfsNodes, kBfsDepth>(t, a, now, q, seen, hole);
-      if (end < 0) break;  // no cuckoo path within the search bound: FULL
-      const int r = execute_path_warp(t, tid, q, end, hole, k, v, a, now, expiry, ws);
-      __syncwarp();  // every lane is done with the queue
-      if (r != 0) {
-        st = r > 0 ? kStInserted : kStBusy;
-        break;
-      }
-    }
+    const uint8_t st = search_warp<kBfsNodes, kBfsDepth>(t, tid, k, v, a, now, expiry, ws, q, seen);
     if (lane == 0) {
       if (st == kStFull && retry) {
         retry[atomicAdd(retry_count, 1u)] = i;
@@ -1329,24 +1334,90 @@ __global__ void __launch_bounds__(kThreads) insert_fixup_finish(TableSet ts, con
                      (uint64_t)gridDim.x * blockDim.x);
 }
 
+// What a small batch's cluster leaves (kClusterFirst below): the searches of the
+// keys that the one-move pass could not place, one warp per key, each going on to
+// the next width by itself, and then, in the last block to finish, the finishing
+// pass. A launch of its own because the widest search takes 50 us if it fails and
+// a cluster has room for few at a time: 256 keys bound for a full table take 0.1
+// ms by these two launches, 12.7 ms when the cluster ran all passes, 0.12 ms as a
+// chain; 2048 keys 0.21, 6.6 and 0.19 ms. It costs batches that leave nothing 1.2
+// to 1.6 us.
+constexpr unsigned kRestBlocksPerSm = 6;  // 32 KB of queue and visited set each
+constexpr int kRestThreads = 128;  // one warp searches, all take part in the finishing pass
+__global__ void __launch_bounds__(kRestThreads) insert_rest(TableSet ts, const uint8_t* __restrict__ keys,
+                                                            const uint64_t* __restrict__ vals, uint32_t now,
+                                                            uint32_t expiry, uint8_t* __restrict__ status,
+                                                            Workspace ws) {
+  __shared__ Node queue[2048];
+  __shared__ uint32_t seen[WarpSeen<2048>::kSize];
+  __shared__ bool last;
+  pdl_wait();
+  const uint32_t listed = ld32_cg(ws.counters + kCntMoved1), blocks = min(gridDim.x, listed);
+  if (blockIdx.x >= blocks) return;
+  if (threadIdx.x < 32) {
+    for (uint32_t j = blockIdx.x; j < listed; j += blocks) {
+      const uint32_t i = ws.retry[j];
+      const TableView t = ts.of(i);
+      const uint32_t tid = ts.id(i);
+      const uint64_t v = load_val(vals, i);
+      const Key k = load_key(keys, i);
+      const Addr a = address_of(k, t.nb, t.seed);
+      uint8_t st = search_warp<96, 4>(t, tid, k, v, a, now, expiry, ws, queue, seen);
+      if (st == kStFull) {
+        if (threadIdx.x == 0) atomicAdd(ws.counters + kCntGrid, 1u);
+        st = search_warp<192, 5>(t, tid, k, v, a, now, expiry, ws, queue, seen);
+      }
+      if (st == kStFull) {
+        uint32_t taken = 0;
+        if (threadIdx.x == 0) taken = atomicAdd(ws.counters + kCntSecond, 1u);
+        if (__shfl_sync(kWarpAll, taken, 0) < kLastPassKeys)
+          st = search_warp<2048, 6>(t, tid, k, v, a, now, expiry, ws, queue, seen);
+      }
+      if (threadIdx.x == 0) {
+        if (st == kStBusy) latch_error(t, kErrLockTimeout);
+        status[i] = st;
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    fence_acq_rel();
+    last = atomicAdd(ws.counters + kCntRest, 1u) == blocks - 1;
+    fence_acq_rel();
+  }
+  __syncthreads();
+  if (last) fixup_finish_range(ts, keys, vals, status, ws, load_counts(ws), threadIdx.x, kRestThreads);
+}
+
 // --------------------------------------------------- single-launch insert
-// The whole insert call in one launch, the stages of the chain above in order
-// with a barrier between them instead of a kernel boundary. A stage whose list
-// is empty is skipped with its barrier. Two forms:
-//   a cluster     (the default for small batches) one cluster of up to eight
-//                 blocks, which clears the workspace as well: a small batch
-//                 spends most of a chain's time in the starts and drains of the
-//                 chain's eight dependent launches, each also 1.9 us of host
-//                 time, and a cluster's barrier takes a fraction of either;
+// The stages of the chain above in one launch, in order, with a barrier between
+// them instead of a kernel boundary. A stage whose list is empty is skipped with
+// its barrier. Three forms:
+//   a whole cluster  (at most 64 keys) eight blocks of one cluster run the whole
+//                 call. The first one works alone until there are keys without a
+//                 slot, with the set and the groups of equal keys in shared
+//                 memory (an update of 64 keys 5.7 us, 6.4 with the set in the
+//                 workspace and all blocks at work); the others are there for
+//                 the searches, 48 of the widest at a time;
+//   a cluster first  (up to 2048 keys) one cluster of up to eight blocks runs the
+//                 stages up to the one-move pass, and the finishing pass if that
+//                 leaves nothing; insert_rest, launched after it, the rest.
+//                 Small batches spend most of a chain's time in the starts and
+//                 drains of its seven dependent launches, each also 1.9 us of
+//                 host time, and a cluster's barrier takes a fraction of either;
 //   a whole grid  (CKPP_INSERT_LAUNCH_SINGLE, any size) a cooperative launch
 //                 on a grid sized to the batch, after the workspace clear. All
 //                 blocks are resident at once, so the barrier cannot wait on a
 //                 block that has not started.
-// Search queues live in 48 KB of dynamic shared memory per block: the
+// Search queues live in dynamic shared memory (48 KB per block of a grid): the
 // grid pass runs on 64 threads of every block (96 nodes each; on every warp
-// for a short list), the second pass
-// on every warp (192 nodes and a visited set each), the last on the first warp
-// of every block (2048 nodes and the visited set).
+// for a short list), the second pass on every warp (192 nodes and a visited set
+// each), the last (2048 nodes and the visited set) on the first warp of every
+// block, or on six warps of a whole cluster's blocks.
+enum SingleForm : int { kWholeGrid, kWholeCluster, kClusterFirst };
+// The largest batch that a whole cluster takes on: 64 keys bound for a full table,
+// two rounds of the widest search, take 150 us, a chain 115; 32 keys 104 and 114.
+constexpr uint64_t kWholeKeys = 64;
 constexpr int kSingleThreads = 256;
 constexpr size_t kSingleSmem = 48 * 1024;
 constexpr unsigned kSingleMinBlocks = 8;
@@ -1399,10 +1470,10 @@ __device__ bool grid_barrier(uint32_t* count, uint32_t* gen) {
   return ok_s != 0;
 }
 
-// The barrier between two stages of either form.
-template <bool kCluster>
+// The barrier between two stages.
+template <SingleForm kForm>
 __device__ __forceinline__ bool stage_barrier(const Workspace& ws) {
-  if constexpr (kCluster) {
+  if constexpr (kForm != kWholeGrid) {
     cluster_barrier();
     return true;
   } else {
@@ -1410,52 +1481,62 @@ __device__ __forceinline__ bool stage_barrier(const Workspace& ws) {
   }
 }
 
-// A cluster of one block keeps the set and the groups of equal keys in shared
-// memory: the set before the queues need the room, the groups behind them.
-constexpr size_t kOneSetAt = 20 * 1024, kOneGroupsAt = kSingleSmem - sizeof(OneBlockGroups);
+// Where a block that works alone keeps the set and the groups of equal keys: the
+// set before the queues need the room, the groups behind them.
+constexpr unsigned kWholeBlocks = 8;
+constexpr uint32_t kWholeWidest = 6;  // warps of a whole cluster's block that run the last pass
+constexpr size_t kQueueBytes = kSingleSmem - sizeof(OneBlockGroups);
+constexpr size_t kWholeQueueBytes = kWholeWidest * warp_search_bytes<2048>();
+constexpr size_t kWholeSmem = kWholeQueueBytes + sizeof(OneBlockGroups);
+constexpr size_t kOneSetAt = 20 * 1024;
 static_assert((kSingleThreads / 32) * sizeof(P1Rows) + sizeof(P1Lists) <= kOneSetAt &&
-                  kOneSetAt + sizeof(OneBlockSet) <= kOneGroupsAt &&
-                  (kSingleThreads / 32) * warp_search_bytes<192>() <= kOneGroupsAt &&
-                  (kSingleThreads / 32) * warp_search_bytes<96>() <= kOneGroupsAt &&
-                  warp_search_bytes<2048>() <= kOneGroupsAt && kOneBlockKeys <= kGridWarpKeys,
+                  kOneSetAt + sizeof(OneBlockSet) <= kQueueBytes &&
+                  (kSingleThreads / 32) * warp_search_bytes<192>() <= kQueueBytes &&
+                  (kSingleThreads / 32) * warp_search_bytes<96>() <= kQueueBytes && kQueueBytes <= kWholeQueueBytes &&
+                  kOneBlockKeys <= kGridWarpKeys,
               "one block's set and groups do not fit beside the queues");
 static_assert(kOneBlockKeys == kSingleThreads, "cluster_blocks gives batches that fit one block a cluster of one");
+static_assert(kWholeKeys <= kOneBlockKeys, "a whole cluster's batch fits its first block");
 
-template <bool kCluster, bool kTimers>
-__global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableSet ts, const uint8_t* __restrict__ keys,
-                                                                         const uint64_t* __restrict__ vals, uint64_t n,
-                                                                         uint32_t now, uint32_t expiry,
-                                                                         uint8_t* __restrict__ status,
-                                                                         Workspace caller_ws) {
+template <SingleForm kForm, bool kTimers>
+__global__ void __launch_bounds__(kSingleThreads, kForm == kWholeCluster ? 1 : 2)
+    insert_single_launch(TableSet ts, const uint8_t* __restrict__ keys, const uint64_t* __restrict__ vals, uint64_t n,
+                         uint32_t now, uint32_t expiry, uint8_t* __restrict__ status, Workspace caller_ws) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t tid = blockIdx.x * kSingleThreads + threadIdx.x;
   const uint32_t threads = gridDim.x * kSingleThreads;
-  const Workspace ws = kCluster && gridDim.x == 1
-                           ? in_shared(caller_ws, *reinterpret_cast<OneBlockSet*>(smem + kOneSetAt),
-                                       *reinterpret_cast<OneBlockGroups*>(smem + kOneGroupsAt))
-                           : caller_ws;
+  // the threads that share phase 1 and the finishing pass: one block's or all
+  const bool one = kForm == kWholeCluster || (kForm == kClusterFirst && gridDim.x == 1);
+  const uint32_t own_threads = one ? kSingleThreads : threads;
+  const Workspace ws =
+      one ? in_shared(caller_ws, *reinterpret_cast<OneBlockSet*>(smem + kOneSetAt),
+                      *reinterpret_cast<OneBlockGroups*>(smem + (kForm == kWholeCluster ? kWholeQueueBytes : kQueueBytes)))
+          : caller_ws;
   bool ok = true;
   pdl_wait();
-  if (kCluster) {
-    clear_workspace(ws, tid, threads);
-    stage_barrier<kCluster>(ws);
+  if (kForm != kWholeCluster || blockIdx.x == 0) {
+    if (kForm != kWholeGrid) {
+      clear_workspace(ws, tid, own_threads);
+      if (kForm == kWholeCluster) {
+        __syncthreads();
+      } else {
+        stage_barrier<kForm>(ws);
+      }
+    }
+    P1Rows* rows = reinterpret_cast<P1Rows*>(smem);  // phase 1's part of the shared memory, before the queues'
+    P1Lists& lists = *reinterpret_cast<P1Lists*>(rows + kSingleThreads / 32);
+    lists_init(lists);
+    for (uint64_t first = blockIdx.x * (uint64_t)kSingleThreads; first < n; first += own_threads) {  // whole blocks
+      const uint64_t i = first + threadIdx.x;
+      phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
+    }
   }
-  P1Rows* rows = reinterpret_cast<P1Rows*>(smem);  // phase 1's part of the shared memory, before the queues'
-  P1Lists& lists = *reinterpret_cast<P1Lists*>(rows + kSingleThreads / 32);
-  lists_init(lists);
-  for (uint64_t first = blockIdx.x * (uint64_t)kSingleThreads; first < n; first += threads) {  // whole blocks
-    const uint64_t i = first + threadIdx.x;
-    phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
-  }
-  ok &= stage_barrier<kCluster>(ws);
+  ok &= stage_barrier<kForm>(ws);
   // lists as in the chain: pending -> one move -> retry -> grid search -> pending -> second pass ->
   // retry -> last pass. A pass whose list is empty is skipped with its barrier, and so are the ones
   // after it; every block reads the same counts (final before the barrier), so all skip alike.
   Counts counts = load_counts(ws);
   if (counts[kCntPending]) {
-    Node* nodes = reinterpret_cast<Node*>(smem);
-    const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kSingleThreads / 32) + w;
-    const uint32_t warps = gridDim.x * (kSingleThreads / 32);
     if (counts[kCntPending] <= min(kMoveHalfKeys, threads / 16u)) {
       move1_range_half(ts, keys, vals, now, expiry, status, ws, ws.pending, counts[kCntPending], ws.retry,
                        ws.counters + kCntMoved1, tid / 16u, threads / 16u);
@@ -1463,40 +1544,58 @@ __global__ void __launch_bounds__(kSingleThreads, 2) insert_single_launch(TableS
       move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, counts[kCntPending], ws.retry,
                   ws.counters + kCntMoved1, tid, threads);
     }
-    ok &= stage_barrier<kCluster>(ws);
+    ok &= stage_barrier<kForm>(ws);
     counts = load_counts(ws);
-    if (const uint32_t listed = counts[kCntMoved1]) {
-      if (listed <= kGridWarpKeys) {  // a short list: one warp per key
-        uint8_t* mine = smem + w * warp_search_bytes<96>();
-        phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                                 ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
-                                 reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)), warp, warps);
-      } else if (threadIdx.x < 64) {
-        const Queue q{nodes + threadIdx.x, 64};
-        phase2_range<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                            ws.counters + kCntGrid, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
+    if (kForm == kClusterFirst) {
+      if (counts[kCntMoved1]) {  // insert_rest goes on from here
+        if (one) {
+          for (uint32_t j = threadIdx.x; j < ws.n; j += kSingleThreads) caller_ws.range[j] = ws.range[j];
+          for (uint32_t j = threadIdx.x; j < counts[kCntFollowers]; j += kSingleThreads)
+            caller_ws.followers[j] = ws.followers[j];
+        }
+        return;
       }
-      ok &= stage_barrier<kCluster>(ws);
-      counts = load_counts(ws);
-    }
-    if (const uint32_t listed = counts[kCntGrid]) {
-      uint8_t* mine = smem + w * warp_search_bytes<192>();
-      phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, listed, ws.retry,
-                                ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
-                                reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)), warp, warps);
-      ok &= stage_barrier<kCluster>(ws);
-      counts = load_counts(ws);
-    }
-    if (const uint32_t listed = counts[kCntSecond]) {
-      if (w == 0)
-        phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, (uint32_t*)nullptr,
-                                   (uint32_t*)nullptr, kLastPassKeys, nodes,
-                                   reinterpret_cast<uint32_t*>(smem + 2048 * sizeof(Node)), blockIdx.x, gridDim.x);
-      ok &= stage_barrier<kCluster>(ws);
-      counts = load_counts(ws);
+    } else {
+      Node* nodes = reinterpret_cast<Node*>(smem);
+      const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kSingleThreads / 32) + w;
+      const uint32_t warps = gridDim.x * (kSingleThreads / 32);
+      if (const uint32_t listed = counts[kCntMoved1]) {
+        if (kForm == kWholeCluster || listed <= kGridWarpKeys) {  // a short list: one warp per key
+          uint8_t* mine = smem + w * warp_search_bytes<96>();
+          phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
+                                   ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
+                                   reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)), warp, warps);
+        } else if (threadIdx.x < 64) {
+          const Queue q{nodes + threadIdx.x, 64};
+          phase2_range<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
+                              ws.counters + kCntGrid, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
+        }
+        ok &= stage_barrier<kForm>(ws);
+        counts = load_counts(ws);
+      }
+      if (const uint32_t listed = counts[kCntGrid]) {
+        uint8_t* mine = smem + w * warp_search_bytes<192>();
+        phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, listed, ws.retry,
+                                  ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
+                                  reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)), warp, warps);
+        ok &= stage_barrier<kForm>(ws);
+        counts = load_counts(ws);
+      }
+      if (const uint32_t listed = counts[kCntSecond]) {
+        constexpr uint32_t kWidest = kForm == kWholeCluster ? kWholeWidest : 1;
+        uint8_t* mine = smem + w * warp_search_bytes<2048>();
+        if (w < kWidest)  // the first keys to different blocks
+          phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, (uint32_t*)nullptr,
+                                     (uint32_t*)nullptr, kLastPassKeys, reinterpret_cast<Node*>(mine),
+                                     reinterpret_cast<uint32_t*>(mine + 2048 * sizeof(Node)),
+                                     w * gridDim.x + blockIdx.x, kWidest * gridDim.x);
+        ok &= stage_barrier<kForm>(ws);
+        counts = load_counts(ws);
+      }
     }
   }
-  fixup_finish_range(ts, keys, vals, status, ws, counts, tid, threads);
+  if (kForm != kWholeCluster || blockIdx.x == 0)
+    fixup_finish_range(ts, keys, vals, status, ws, counts, tid, own_threads);
   if (!ok && threadIdx.x == 0) latch_error(ts.table(0), kErrLockTimeout);
 }
 
@@ -1535,7 +1634,7 @@ int single_launch_blocks_per_sm() {
   if (v) return v > 0 ? v : 0;
   int coop = 0, per_sm = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, insert_single_launch<false, true>, kSingleThreads,
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, insert_single_launch<kWholeGrid, true>, kSingleThreads,
                                                     kSingleSmem) !=
           cudaSuccess) {
     cudaGetLastError();
@@ -1546,6 +1645,24 @@ int single_launch_blocks_per_sm() {
           : -1;
   cache[dev].store(v, std::memory_order_relaxed);
   return v > 0 ? v : 0;
+}
+
+// Allows the whole cluster's shared memory, once per device.
+cudaError_t allow_whole_cluster() {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<bool> done[kMaxDevices];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev >= 0 && dev < kMaxDevices;
+  if (known && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(insert_single_launch<kWholeCluster, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kWholeSmem)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(insert_single_launch<kWholeCluster, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kWholeSmem)) != cudaSuccess)
+    return e;
+  if (known) done[dev].store(true, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 cudaError_t launch_single(const TableSet& ts, const uint8_t* keys, const uint64_t* vals, uint64_t n, uint32_t now,
@@ -1563,7 +1680,7 @@ cudaError_t launch_single(const TableSet& ts, const uint8_t* keys, const uint64_
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, insert_single_launch<false, true>, ts, keys, vals, n, now, expiry, status, ws);
+  return cudaLaunchKernelEx(&cfg, insert_single_launch<kWholeGrid, true>, ts, keys, vals, n, now, expiry, status, ws);
 }
 
 }  // namespace
@@ -1583,10 +1700,20 @@ cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_
       e = launch_workspace_clear(ws, s);
       return e != cudaSuccess ? e : launch_single(ts, keys, vals, n, now, expiry, status, ws, s, per_sm);
     }
+  } else if (n <= kWholeKeys) {
+    if ((e = allow_whole_cluster()) != cudaSuccess) return e;
+    return launch_cluster(ts.any_timers ? insert_single_launch<kWholeCluster, true>
+                                        : insert_single_launch<kWholeCluster, false>,
+                          kWholeBlocks, kSingleThreads, kWholeSmem, s, ts, keys, vals, n, now, expiry, status, ws);
   } else if (n <= kClusterKeys) {
-    return launch_cluster(ts.any_timers ? insert_single_launch<true, true> : insert_single_launch<true, false>,
-                          cluster_blocks(n, kSingleThreads), kSingleThreads, kSingleSmem, s, ts, keys, vals, n, now,
-                          expiry, status, ws);
+    e = launch_cluster(ts.any_timers ? insert_single_launch<kClusterFirst, true>
+                                     : insert_single_launch<kClusterFirst, false>,
+                       cluster_blocks(n, kSingleThreads), kSingleThreads, kSingleSmem, s, ts, keys, vals, n, now, expiry,
+                       status, ws);
+    if (e != cudaSuccess) return e;
+    const unsigned most = kRestBlocksPerSm * (unsigned)device_sm_count();
+    return launch_chained(insert_rest, n < most ? (unsigned)n : most, kRestThreads, s, ts, keys, vals, now, expiry, status,
+                          ws);
   }
   e = launch_workspace_clear(ws, s);
   if (e != cudaSuccess) return e;

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kDirectThreads) lookup_direct_kernel(TableView
 // but each its own DRAM access once the line has gone. 4M keys, all known, load
 // 0.3 / 0.5 / 0.9, lookup_kernel -> this one in us: 240 MB 78 -> 61 / 90 -> 68 /
 // 116 -> 101 (with timers 96 -> 76 / 108 -> 83 / 137 -> 111), 248 MB 79 -> 89 /
-// 90 -> 97 / 117 -> 104, 256 MB 79 -> 100 / 90 -> 103 / 117 -> 104 (with timers
+// 90 -> 97 / 117 -> 102, 256 MB 79 -> 100 / 90 -> 103 / 117 -> 104 (with timers
 // 96 -> 132 / 110 -> 131 / 139 -> 114). Tables that take turns, 512 MB or more
 // in all, gain as much up to 240 MB each. A lookup that refreshes its hits keeps
 // to lookup_kernel: the refresh's store follows three reads of the bucket instead
