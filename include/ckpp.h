@@ -283,11 +283,11 @@ int ckpp_bulk_insert(ckpp_table* table, const ckpp_key* keys, const uint64_t* va
  *                              keys runs the same stages on one thread-block
  *                              cluster, with one launch after it (for more than
  *                              64 keys) for the searches that are left;
- *   CKPP_INSERT_LAUNCH_SINGLE  one cooperative launch running the same stages
- *                              separated by grid-wide barriers, sized to the
- *                              batch, with stages that have nothing to do
- *                              skipped (a device without cooperative launch
- *                              uses the chain).
+ *   CKPP_INSERT_LAUNCH_SINGLE  kept for callers that set it: the chain for every
+ *                              batch size, small ones too. (One cooperative
+ *                              launch with grid-wide barriers was meant by it;
+ *                              measured, it is slower than the chain from 128K
+ *                              keys on and than the cluster below 2048.)
  * The mode is process-wide; set it while no insert call is being issued.
  * Returns the previous mode, or CKPP_EINVAL for an unknown one. */
 #define CKPP_INSERT_LAUNCH_CHAIN 0
@@ -310,7 +310,7 @@ int ckpp_bulk_delete(ckpp_table* table, const ckpp_key* keys, uint64_t n, uint32
 /* Bulk insert for callers that cannot allocate device memory. No counterpart
  * in the paper: it is ckpp_bulk_insert with the same semantics, arguments and
  * status codes, minus the workspace. Its scratch is a fixed device array built
- * into libckpp.so (about 6 MB, enough for CKPP_NOALLOC_MAX_KEYS keys), which
+ * into libckpp.so (about 4.5 MB, enough for CKPP_NOALLOC_MAX_KEYS keys), which
  * every GPU that loads the library holds until the process exits. It suits
  * callers that own no allocator when they insert: a data-plane thread that must
  * never call cudaMalloc/cudaFree (cudaFree can stall the whole device), or a

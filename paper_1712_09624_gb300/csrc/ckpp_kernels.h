@@ -42,8 +42,7 @@ constexpr uint32_t kCntFollowers = 4;      // repeated keys (in `followers`)
 constexpr uint32_t kCntGrid = 5;           // keys the grid search left (in `pending`)
 constexpr uint32_t kCntSecond = 6;         // keys the second search left (in `retry`)
 constexpr uint32_t kCntSticky = 7;         // claimed bits to clear (in `sticky`)
-constexpr uint32_t kCntBarrier = 8;        // two words: the grid barrier of the single-launch insert
-constexpr uint32_t kCntRest = 10;          // blocks of the launch after a small batch's cluster that are done
+constexpr uint32_t kCntRest = 8;           // blocks of the launch after a small batch's cluster that are done
 constexpr uint32_t kCounterWords = 64;
 
 // Device scratch for one insert or delete batch (carved out of the caller's
@@ -109,8 +108,7 @@ cudaError_t launch_batched_lookup(const TableView* tables, uint32_t n_tables, co
 // launch.
 cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s);
 
-// An insert call runs as a chain of kernels (the default) or as one
-// cooperative launch (insert.cu), whichever mode the caller picks.
+// The insert launch modes a caller can pick (insert.cu).
 constexpr int kInsertLaunchChain = 0, kInsertLaunchSingle = 1;
 int set_insert_launch(int mode);  // returns the previous mode, or -1 for an unknown mode
 

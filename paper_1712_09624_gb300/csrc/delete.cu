@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kSettleThreads) delete_settle(uint8_t* __restr
   settle_range(status, ws, ld32_cg(ws.counters + kCntFollowers), blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-// A small batch in one launch of one cluster (as insert_single_launch).
+// A small batch in one launch of one cluster (as insert_cluster).
 template <int kTM>
 __global__ void __launch_bounds__(kDeleteClusterThreads) delete_cluster(TableSet ts, const uint8_t* __restrict__ keys,
                                                                  uint64_t n, uint32_t now,

@@ -1334,7 +1334,7 @@ __global__ void __launch_bounds__(kThreads) insert_fixup_finish(TableSet ts, con
                      (uint64_t)gridDim.x * blockDim.x);
 }
 
-// What a small batch's cluster leaves (kClusterFirst below): the searches of the
+// What a small batch's cluster leaves (insert_cluster<false> below): the searches of the
 // keys that the one-move pass could not place, one warp per key, each going on to
 // the next width by itself, and then, in the last block to finish, the finishing
 // pass. A launch of its own because the widest search takes 50 us if it fails and
@@ -1389,214 +1389,131 @@ __global__ void __launch_bounds__(kRestThreads) insert_rest(TableSet ts, const u
   if (last) fixup_finish_range(ts, keys, vals, status, ws, load_counts(ws), threadIdx.x, kRestThreads);
 }
 
-// --------------------------------------------------- single-launch insert
-// The stages of the chain above in one launch, in order, with a barrier between
-// them instead of a kernel boundary. A stage whose list is empty is skipped with
-// its barrier. Three forms:
-//   a whole cluster  (at most 64 keys) eight blocks of one cluster run the whole
-//                 call. The first one works alone until there are keys without a
-//                 slot, with the set and the groups of equal keys in shared
-//                 memory (an update of 64 keys 5.7 us, 6.4 with the set in the
-//                 workspace and all blocks at work); the others are there for
-//                 the searches, 48 of the widest at a time;
-//   a cluster first  (up to 2048 keys) one cluster of up to eight blocks runs the
-//                 stages up to the one-move pass, and the finishing pass if that
-//                 leaves nothing; insert_rest, launched after it, the rest.
-//                 Small batches spend most of a chain's time in the starts and
-//                 drains of its seven dependent launches, each also 1.9 us of
-//                 host time, and a cluster's barrier takes a fraction of either;
-//   a whole grid  (CKPP_INSERT_LAUNCH_SINGLE, any size) a cooperative launch
-//                 on a grid sized to the batch, after the workspace clear. All
-//                 blocks are resident at once, so the barrier cannot wait on a
-//                 block that has not started.
-// Search queues live in dynamic shared memory (48 KB per block of a grid): the
-// grid pass runs on 64 threads of every block (96 nodes each; on every warp
-// for a short list), the second pass on every warp (192 nodes and a visited set
-// each), the last (2048 nodes and the visited set) on the first warp of every
-// block, or on six warps of a whole cluster's blocks.
-enum SingleForm : int { kWholeGrid, kWholeCluster, kClusterFirst };
-// The largest batch that a whole cluster takes on: 64 keys bound for a full table,
-// two rounds of the widest search, take 150 us, a chain 115; 32 keys 104 and 114.
+// --------------------------------------------------------- small batches
+// The stages of the chain above on one cluster, in order, with a cluster barrier
+// between them instead of a kernel boundary: a small batch spends most of a
+// chain's time in the starts and drains of its seven dependent launches, each
+// also 1.9 us of host time, and a cluster's barrier takes a fraction of either. A
+// stage whose list is empty is skipped with its barrier. Two forms:
+//   whole (at most 64 keys)  eight blocks of one cluster run the whole call. The
+//         first one works alone until there are keys without a slot, with the set
+//         and the groups of equal keys in shared memory (an update of 64 keys 5.7
+//         us, 6.4 with the set in the workspace and all blocks at work); the
+//         others are there for the searches, 48 of the widest at a time;
+//   first (up to 2048 keys)  one cluster of up to eight blocks runs the stages up
+//         to the one-move pass, and the finishing pass if that leaves nothing;
+//         insert_rest, launched after it, the rest. A batch that fits one block
+//         has one, with the set and the groups in shared memory.
+// The whole form's search queues take the place of phase 1's shared memory: the
+// grid and the second pass run on every warp (96 and 192 nodes and a visited set
+// each), the last (2048 nodes and the visited set) on six warps of every block.
+// The largest batch of the whole form: 64 keys bound for a full table, two rounds
+// of the widest search, take 150 us, a chain 115; 32 keys 104 and 114.
 constexpr uint64_t kWholeKeys = 64;
-constexpr int kSingleThreads = 256;
-constexpr size_t kSingleSmem = 48 * 1024;
-constexpr unsigned kSingleMinBlocks = 8;
-// Bounded wait at a barrier: about 2-4 s of polls (each a load and a 64 ns sleep), longer than
-// the bounded lock waits a stage may contain, so a barrier gives up only if a block never arrives.
-constexpr int kBarrierSpins = 1 << 22;
-
-static_assert((kSingleThreads / 32) * sizeof(P1Rows) + sizeof(P1Lists) <= kSingleSmem, "phase 1 rows exceed the shared memory");
-static_assert(96 * 64 * sizeof(Node) <= kSingleSmem, "grid pass queues exceed the shared memory");
-static_assert((kSingleThreads / 32) * warp_search_bytes<96>() <= kSingleSmem,
-              "grid pass state (one warp per key) exceeds the shared memory");
-static_assert((kSingleThreads / 32) * warp_search_bytes<192>() <= kSingleSmem,
-              "second pass state exceeds the shared memory");
-static_assert(warp_search_bytes<2048>() <= kSingleSmem, "last pass state exceeds the shared memory");
-
-__device__ __forceinline__ uint32_t ld_acquire32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Grid-wide barrier over gridDim.x resident blocks. count and gen are two
-// words of the workspace's zeroed counters: every block reads the generation,
-// then arrives on the count; the last to arrive resets the count and advances
-// the generation (release), and the others wait for it (acquire). Returns
-// false if the wait gave up after kBarrierSpins polls.
-__device__ bool grid_barrier(uint32_t* count, uint32_t* gen) {
-  __shared__ int ok_s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");  // this block's writes before the arrival
-    const uint32_t g = ld_acquire32(gen);
-    if (atomicAdd(count, 1u) == gridDim.x - 1) {
-      atomicExch(count, 0u);
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gen) : "memory");
-    } else {
-      for (int spin = 0; ld_acquire32(gen) == g; ++spin) {
-        if (spin >= kBarrierSpins) {
-          ok = 0;
-          break;
-        }
-        __nanosleep(64);
-      }
-    }
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");  // the other blocks' writes after it
-    ok_s = ok;
-  }
-  __syncthreads();
-  return ok_s != 0;
-}
-
-// The barrier between two stages.
-template <SingleForm kForm>
-__device__ __forceinline__ bool stage_barrier(const Workspace& ws) {
-  if constexpr (kForm != kWholeGrid) {
-    cluster_barrier();
-    return true;
-  } else {
-    return grid_barrier(ws.counters + kCntBarrier, ws.counters + kCntBarrier + 1);
-  }
-}
-
-// Where a block that works alone keeps the set and the groups of equal keys: the
-// set before the queues need the room, the groups behind them.
 constexpr unsigned kWholeBlocks = 8;
-constexpr uint32_t kWholeWidest = 6;  // warps of a whole cluster's block that run the last pass
-constexpr size_t kQueueBytes = kSingleSmem - sizeof(OneBlockGroups);
-constexpr size_t kWholeQueueBytes = kWholeWidest * warp_search_bytes<2048>();
-constexpr size_t kWholeSmem = kWholeQueueBytes + sizeof(OneBlockGroups);
+constexpr uint32_t kWholeWidest = 6;  // warps of a block that run the last pass
+constexpr int kClusterThreads = 256;
+// Shared memory: phase 1's rows and lists, then the set; the queues over both; the
+// groups, which the finishing pass reads, behind.
 constexpr size_t kOneSetAt = 20 * 1024;
-static_assert((kSingleThreads / 32) * sizeof(P1Rows) + sizeof(P1Lists) <= kOneSetAt &&
-                  kOneSetAt + sizeof(OneBlockSet) <= kQueueBytes &&
-                  (kSingleThreads / 32) * warp_search_bytes<192>() <= kQueueBytes &&
-                  (kSingleThreads / 32) * warp_search_bytes<96>() <= kQueueBytes && kQueueBytes <= kWholeQueueBytes &&
-                  kOneBlockKeys <= kGridWarpKeys,
-              "one block's set and groups do not fit beside the queues");
-static_assert(kOneBlockKeys == kSingleThreads, "cluster_blocks gives batches that fit one block a cluster of one");
-static_assert(kWholeKeys <= kOneBlockKeys, "a whole cluster's batch fits its first block");
+constexpr size_t kFirstGroupsAt = kOneSetAt + sizeof(OneBlockSet);
+constexpr size_t kFirstSmem = kFirstGroupsAt + sizeof(OneBlockGroups);
+constexpr size_t kWholeGroupsAt = kWholeWidest * warp_search_bytes<2048>();
+constexpr size_t kWholeSmem = kWholeGroupsAt + sizeof(OneBlockGroups);
+static_assert((kClusterThreads / 32) * sizeof(P1Rows) + sizeof(P1Lists) <= kOneSetAt && kFirstSmem <= 48 * 1024 &&
+                  kFirstGroupsAt <= kWholeGroupsAt &&
+                  (kClusterThreads / 32) * warp_search_bytes<192>() <= kWholeGroupsAt &&
+                  (kClusterThreads / 32) * warp_search_bytes<96>() <= kWholeGroupsAt,
+              "the parts of the shared memory overlap");
+static_assert(kOneBlockKeys == kClusterThreads, "cluster_blocks gives batches that fit one block a cluster of one");
+static_assert(kWholeKeys <= kOneBlockKeys, "a whole form's batch fits its first block");
 
-template <SingleForm kForm, bool kTimers>
-__global__ void __launch_bounds__(kSingleThreads, kForm == kWholeCluster ? 1 : 2)
-    insert_single_launch(TableSet ts, const uint8_t* __restrict__ keys, const uint64_t* __restrict__ vals, uint64_t n,
-                         uint32_t now, uint32_t expiry, uint8_t* __restrict__ status, Workspace caller_ws) {
+template <bool kWhole, bool kTimers>
+__global__ void __launch_bounds__(kClusterThreads, kWhole ? 1 : 2)
+    insert_cluster(TableSet ts, const uint8_t* __restrict__ keys, const uint64_t* __restrict__ vals, uint64_t n,
+                   uint32_t now, uint32_t expiry, uint8_t* __restrict__ status, Workspace caller_ws) {
   extern __shared__ __align__(128) uint8_t smem[];
-  const uint32_t tid = blockIdx.x * kSingleThreads + threadIdx.x;
-  const uint32_t threads = gridDim.x * kSingleThreads;
+  const uint32_t tid = blockIdx.x * kClusterThreads + threadIdx.x;
+  const uint32_t threads = gridDim.x * kClusterThreads;
   // the threads that share phase 1 and the finishing pass: one block's or all
-  const bool one = kForm == kWholeCluster || (kForm == kClusterFirst && gridDim.x == 1);
-  const uint32_t own_threads = one ? kSingleThreads : threads;
-  const Workspace ws =
-      one ? in_shared(caller_ws, *reinterpret_cast<OneBlockSet*>(smem + kOneSetAt),
-                      *reinterpret_cast<OneBlockGroups*>(smem + (kForm == kWholeCluster ? kWholeQueueBytes : kQueueBytes)))
-          : caller_ws;
-  bool ok = true;
+  const bool one = kWhole || gridDim.x == 1;
+  const uint32_t own_threads = one ? kClusterThreads : threads;
+  const Workspace ws = one ? in_shared(caller_ws, *reinterpret_cast<OneBlockSet*>(smem + kOneSetAt),
+                                       *reinterpret_cast<OneBlockGroups*>(smem + (kWhole ? kWholeGroupsAt : kFirstGroupsAt)))
+                           : caller_ws;
   pdl_wait();
-  if (kForm != kWholeCluster || blockIdx.x == 0) {
-    if (kForm != kWholeGrid) {
-      clear_workspace(ws, tid, own_threads);
-      if (kForm == kWholeCluster) {
-        __syncthreads();
-      } else {
-        stage_barrier<kForm>(ws);
-      }
+  if (!kWhole || blockIdx.x == 0) {
+    clear_workspace(ws, tid, own_threads);
+    if (kWhole) {
+      __syncthreads();
+    } else {
+      cluster_barrier();
     }
-    P1Rows* rows = reinterpret_cast<P1Rows*>(smem);  // phase 1's part of the shared memory, before the queues'
-    P1Lists& lists = *reinterpret_cast<P1Lists*>(rows + kSingleThreads / 32);
+    P1Rows* rows = reinterpret_cast<P1Rows*>(smem);
+    P1Lists& lists = *reinterpret_cast<P1Lists*>(rows + kClusterThreads / 32);
     lists_init(lists);
-    for (uint64_t first = blockIdx.x * (uint64_t)kSingleThreads; first < n; first += own_threads) {  // whole blocks
+    for (uint64_t first = blockIdx.x * (uint64_t)kClusterThreads; first < n; first += own_threads) {  // whole blocks
       const uint64_t i = first + threadIdx.x;
       phase1_one<kTimers>(ts, keys, vals, now, expiry, status, ws, i, i < n, rows[threadIdx.x >> 5], lists);
     }
   }
-  ok &= stage_barrier<kForm>(ws);
+  cluster_barrier();
   // lists as in the chain: pending -> one move -> retry -> grid search -> pending -> second pass ->
   // retry -> last pass. A pass whose list is empty is skipped with its barrier, and so are the ones
   // after it; every block reads the same counts (final before the barrier), so all skip alike.
   Counts counts = load_counts(ws);
   if (counts[kCntPending]) {
-    if (counts[kCntPending] <= min(kMoveHalfKeys, threads / 16u)) {
+    if (counts[kCntPending] <= threads / 16u) {
       move1_range_half(ts, keys, vals, now, expiry, status, ws, ws.pending, counts[kCntPending], ws.retry,
                        ws.counters + kCntMoved1, tid / 16u, threads / 16u);
     } else {
       move1_range(ts, keys, vals, now, expiry, status, ws, ws.pending, counts[kCntPending], ws.retry,
                   ws.counters + kCntMoved1, tid, threads);
     }
-    ok &= stage_barrier<kForm>(ws);
+    cluster_barrier();
     counts = load_counts(ws);
-    if (kForm == kClusterFirst) {
-      if (counts[kCntMoved1]) {  // insert_rest goes on from here
-        if (one) {
-          for (uint32_t j = threadIdx.x; j < ws.n; j += kSingleThreads) caller_ws.range[j] = ws.range[j];
-          for (uint32_t j = threadIdx.x; j < counts[kCntFollowers]; j += kSingleThreads)
-            caller_ws.followers[j] = ws.followers[j];
-        }
-        return;
-      }
-    } else {
-      Node* nodes = reinterpret_cast<Node*>(smem);
-      const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kSingleThreads / 32) + w;
-      const uint32_t warps = gridDim.x * (kSingleThreads / 32);
-      if (const uint32_t listed = counts[kCntMoved1]) {
-        if (kForm == kWholeCluster || listed <= kGridWarpKeys) {  // a short list: one warp per key
-          uint8_t* mine = smem + w * warp_search_bytes<96>();
-          phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                                   ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
-                                   reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)), warp, warps);
-        } else if (threadIdx.x < 64) {
-          const Queue q{nodes + threadIdx.x, 64};
-          phase2_range<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
-                              ws.counters + kCntGrid, 0xFFFFFFFFu, q, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
-        }
-        ok &= stage_barrier<kForm>(ws);
-        counts = load_counts(ws);
-      }
-      if (const uint32_t listed = counts[kCntGrid]) {
-        uint8_t* mine = smem + w * warp_search_bytes<192>();
-        phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, listed, ws.retry,
-                                  ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
-                                  reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)), warp, warps);
-        ok &= stage_barrier<kForm>(ws);
-        counts = load_counts(ws);
-      }
-      if (const uint32_t listed = counts[kCntSecond]) {
-        constexpr uint32_t kWidest = kForm == kWholeCluster ? kWholeWidest : 1;
-        uint8_t* mine = smem + w * warp_search_bytes<2048>();
-        if (w < kWidest)  // the first keys to different blocks
-          phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, (uint32_t*)nullptr,
-                                     (uint32_t*)nullptr, kLastPassKeys, reinterpret_cast<Node*>(mine),
-                                     reinterpret_cast<uint32_t*>(mine + 2048 * sizeof(Node)),
-                                     w * gridDim.x + blockIdx.x, kWidest * gridDim.x);
-        ok &= stage_barrier<kForm>(ws);
-        counts = load_counts(ws);
-      }
-    }
   }
-  if (kForm != kWholeCluster || blockIdx.x == 0)
+  if constexpr (!kWhole) {
+    if (counts[kCntMoved1]) {  // insert_rest goes on from here
+      if (one) {
+        for (uint32_t j = threadIdx.x; j < ws.n; j += kClusterThreads) caller_ws.range[j] = ws.range[j];
+        for (uint32_t j = threadIdx.x; j < counts[kCntFollowers]; j += kClusterThreads)
+          caller_ws.followers[j] = ws.followers[j];
+      }
+      return;
+    }
     fixup_finish_range(ts, keys, vals, status, ws, counts, tid, own_threads);
-  if (!ok && threadIdx.x == 0) latch_error(ts.table(0), kErrLockTimeout);
+  } else {
+    const uint32_t w = threadIdx.x >> 5, warp = blockIdx.x * (kClusterThreads / 32) + w;
+    const uint32_t warps = gridDim.x * (kClusterThreads / 32);
+    if (const uint32_t listed = counts[kCntMoved1]) {
+      uint8_t* mine = smem + w * warp_search_bytes<96>();
+      phase2_range_warp<96, 4>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, ws.pending,
+                               ws.counters + kCntGrid, 0xFFFFFFFFu, reinterpret_cast<Node*>(mine),
+                               reinterpret_cast<uint32_t*>(mine + 96 * sizeof(Node)), warp, warps);
+      cluster_barrier();
+      counts = load_counts(ws);
+    }
+    if (const uint32_t listed = counts[kCntGrid]) {
+      uint8_t* mine = smem + w * warp_search_bytes<192>();
+      phase2_range_warp<192, 5>(ts, keys, vals, now, expiry, status, ws, ws.pending, listed, ws.retry,
+                                ws.counters + kCntSecond, kSecondPassKeys, reinterpret_cast<Node*>(mine),
+                                reinterpret_cast<uint32_t*>(mine + 192 * sizeof(Node)), warp, warps);
+      cluster_barrier();
+      counts = load_counts(ws);
+    }
+    if (const uint32_t listed = counts[kCntSecond]) {
+      uint8_t* mine = smem + w * warp_search_bytes<2048>();
+      if (w < kWholeWidest)  // the first keys to different blocks
+        phase2_range_warp<2048, 6>(ts, keys, vals, now, expiry, status, ws, ws.retry, listed, (uint32_t*)nullptr,
+                                   (uint32_t*)nullptr, kLastPassKeys, reinterpret_cast<Node*>(mine),
+                                   reinterpret_cast<uint32_t*>(mine + 2048 * sizeof(Node)), w * gridDim.x + blockIdx.x,
+                                   kWholeWidest * gridDim.x);
+      cluster_barrier();
+      counts = load_counts(ws);
+    }
+    if (blockIdx.x == 0) fixup_finish_range(ts, keys, vals, status, ws, counts, tid, own_threads);
+  }
 }
 
 // ------------------------------------------------------- workspace reset
@@ -1618,34 +1535,9 @@ cudaError_t launch_workspace_clear(const Workspace& ws, cudaStream_t s) {
 
 namespace {
 
+// kInsertLaunchSingle, once meant for a cooperative launch of the whole call, runs the
+// chain whatever the batch's size.
 std::atomic<int> g_insert_launch{kInsertLaunchChain};
-
-// Blocks per SM the single-launch kernel reaches (queried once per device; 0 if
-// it cannot run, or the device has too few SMs for its search passes).
-int single_launch_blocks_per_sm() {
-  constexpr int kMaxDevices = 64;
-  static std::atomic<int> cache[kMaxDevices];  // 0 unknown, -1 cannot run, else blocks per SM
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
-    cudaGetLastError();
-    return 0;
-  }
-  int v = cache[dev].load(std::memory_order_relaxed);
-  if (v) return v > 0 ? v : 0;
-  int coop = 0, per_sm = 0;
-  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, insert_single_launch<kWholeGrid, true>, kSingleThreads,
-                                                    kSingleSmem) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  v = (coop && per_sm > 0 && (uint64_t)device_sm_count() * (per_sm < 2 ? per_sm : 2) >= kSingleMinBlocks)
-          ? (per_sm < 2 ? per_sm : 2)
-          : -1;
-  cache[dev].store(v, std::memory_order_relaxed);
-  return v > 0 ? v : 0;
-}
 
 // Allows the whole cluster's shared memory, once per device.
 cudaError_t allow_whole_cluster() {
@@ -1656,31 +1548,13 @@ cudaError_t allow_whole_cluster() {
   if (e != cudaSuccess) return e;
   const bool known = dev >= 0 && dev < kMaxDevices;
   if (known && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
-  if ((e = cudaFuncSetAttribute(insert_single_launch<kWholeCluster, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if ((e = cudaFuncSetAttribute(insert_cluster<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kWholeSmem)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(insert_single_launch<kWholeCluster, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      (e = cudaFuncSetAttribute(insert_cluster<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kWholeSmem)) != cudaSuccess)
     return e;
   if (known) done[dev].store(true, std::memory_order_relaxed);
   return cudaSuccess;
-}
-
-cudaError_t launch_single(const TableSet& ts, const uint8_t* keys, const uint64_t* vals, uint64_t n, uint32_t now,
-                          uint32_t expiry, uint8_t* status, const Workspace& ws, cudaStream_t s, int per_sm) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cudaLaunchConfig_t cfg = {};
-  // one thread per key up to the resident limit, and a few blocks for the warps of the search passes
-  const uint64_t want = (n + kSingleThreads - 1) / kSingleThreads;
-  const uint64_t lo = kSingleMinBlocks, hi = (uint64_t)device_sm_count() * per_sm;
-  cfg.gridDim = dim3((unsigned)(want < lo ? lo : (want > hi ? hi : want)));
-  cfg.blockDim = dim3(kSingleThreads);
-  cfg.dynamicSmemBytes = kSingleSmem;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, insert_single_launch<kWholeGrid, true>, ts, keys, vals, n, now, expiry, status, ws);
 }
 
 }  // namespace
@@ -1692,23 +1566,15 @@ int set_insert_launch(int mode) {
 
 cudaError_t launch_insert(const TableSet& ts, const uint8_t* keys, const uint64_t* vals, uint64_t n, uint32_t now,
                           uint32_t expiry, uint8_t* status, const Workspace& ws, cudaStream_t s) {
-  const int mode = g_insert_launch.load(std::memory_order_relaxed);
   cudaError_t e;
-  if (mode == kInsertLaunchSingle) {
-    const int per_sm = single_launch_blocks_per_sm();
-    if (per_sm > 0) {
-      e = launch_workspace_clear(ws, s);
-      return e != cudaSuccess ? e : launch_single(ts, keys, vals, n, now, expiry, status, ws, s, per_sm);
+  if (n <= kClusterKeys && g_insert_launch.load(std::memory_order_relaxed) != kInsertLaunchSingle) {
+    if (n <= kWholeKeys) {
+      if ((e = allow_whole_cluster()) != cudaSuccess) return e;
+      return launch_cluster(ts.any_timers ? insert_cluster<true, true> : insert_cluster<true, false>, kWholeBlocks,
+                            kClusterThreads, kWholeSmem, s, ts, keys, vals, n, now, expiry, status, ws);
     }
-  } else if (n <= kWholeKeys) {
-    if ((e = allow_whole_cluster()) != cudaSuccess) return e;
-    return launch_cluster(ts.any_timers ? insert_single_launch<kWholeCluster, true>
-                                        : insert_single_launch<kWholeCluster, false>,
-                          kWholeBlocks, kSingleThreads, kWholeSmem, s, ts, keys, vals, n, now, expiry, status, ws);
-  } else if (n <= kClusterKeys) {
-    e = launch_cluster(ts.any_timers ? insert_single_launch<kClusterFirst, true>
-                                     : insert_single_launch<kClusterFirst, false>,
-                       cluster_blocks(n, kSingleThreads), kSingleThreads, kSingleSmem, s, ts, keys, vals, n, now, expiry,
+    e = launch_cluster(ts.any_timers ? insert_cluster<false, true> : insert_cluster<false, false>,
+                       cluster_blocks(n, kClusterThreads), kClusterThreads, kFirstSmem, s, ts, keys, vals, n, now, expiry,
                        status, ws);
     if (e != cudaSuccess) return e;
     const unsigned most = kRestBlocksPerSm * (unsigned)device_sm_count();

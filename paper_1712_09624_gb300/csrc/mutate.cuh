@@ -65,8 +65,7 @@ __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gp
 
 // A bucket lock is held for microseconds (one cuckoo path's moves); a waiter
 // gives up after about 0.2 s of polls with back-off (each poll an atomic and a
-// sleep of up to 1 us), far longer than any holder, and well inside the grid
-// barrier's bound of the single-launch insert.
+// sleep of up to 1 us), far longer than any holder.
 constexpr int kLockSpins = 1 << 17;
 
 __device__ __forceinline__ bool lock_bucket(const TableView& t, uint32_t b, uint32_t& ctrl) {
