@@ -1296,7 +1296,9 @@ __device__ void fixup_finish_range(const TableSet& ts, const uint8_t* __restrict
     const uint2 range = ws.range[f.y];
     const bool last = f.x > f.y && f.x == range.y;  // its value is the one that stays (y of 0: none above the owner)
     // The buckets of a last occurrence are requested before the owner's outcome is looked at, both
-    // at once where there are so few that the time of one counts and not their requests.
+    // at once where there are so few that the time of one counts and not their requests. (Both at
+    // once / one after the other: cycles of 32K keys, 90 % of them repeated, 38.3 / 39.7 us; of 256K,
+    // 30 %, 82.2 / 81.3, and 1M 251.6 / 247.7.)
     TableView t{};
     Addr a{};
     Snap s1{}, s2{};
